@@ -390,9 +390,9 @@ static PsumLayout psum_layout(const TTV& U, const TTV& Z, bool bwd) {
     o += align256(sizeof(float) * nL);
     l.offW = o;
     o += align256(sizeof(float) * l.gsize);
-    if (psweep_supported(U, Z)) {  // transposed V, U, W for the right sweep and the gradients
+    if (psweep_supported(U, Z)) {  // slice-major U, V, W in both orientations
       l.offXT = o;
-      o += align256(sizeof(float) * 3 * xtranspose_offsets(U, nullptr));
+      o += align256(sizeof(float) * 6 * xslices_size(U));
     }
     l.jchunk = 0;
     l.nchunks = 0;
@@ -403,8 +403,8 @@ static PsumLayout psum_layout(const TTV& U, const TTV& Z, bool bwd) {
     l.offPart = o;
     o += align256(sizeof(float) * l.gsize * l.nchunks);
     l.offP = l.offQ = l.offW = 0;
-    l.offXT = o;  // transposed V for the right sweep
-    o += align256(sizeof(float) * xtranspose_offsets(U, nullptr));
+    l.offXT = o;  // slice-major U (left sweep) and V (right sweep)
+    o += align256(sizeof(float) * 2 * xslices_size(U));
     if (psweep_tc_supported(U, Z)) {  // operand images of the TF32 sweeps
       l.offImg = o;
       o += align256(psweep_tc_img_bytes(U));
@@ -472,14 +472,12 @@ extern "C" t3f_status t3f_project_sum(const t3f_tt* U, const t3f_tt* V, const t3
   if (psweep_supported(vu, vz)) {
     int* err = static_cast<int*>(ws);
     if (cudaMemsetAsync(ws, 0, sizeof(int), s) != cudaSuccess) return T3F_ERR_CUDA;
-    T3F_CHECK(run_psweep(vu, vz, 0, static_cast<const float*>(vu.p), nullptr, nullptr, Lst, nullptr, l.ioffL, s, err));
-    // the right sweep stages its slices from a transposed copy of V (16-byte copies)
-    float* VT = reinterpret_cast<float*>(w + l.offXT);
-    long long toff[T3F_MAX_D];
-    xtranspose_offsets(vv, toff);
-    const float* vsrc[1] = {static_cast<const float*>(vv.p)};
-    T3F_CHECK(run_xtranspose(vv, vsrc, 1, VT, s));
-    T3F_CHECK(run_psweep(vv, vz, 1, VT, nullptr, nullptr, Rst, nullptr, l.ioffR, s, err, toff));
+    // both sweeps bring their slices in by bulk copies of slice-major copies of U and V
+    float* XC = reinterpret_cast<float*>(w + l.offXT);
+    const float* srcs[2] = {static_cast<const float*>(vu.p), static_cast<const float*>(vv.p)};
+    T3F_CHECK(run_xslices(vu, srcs, 2u, 2, XC, s));
+    T3F_CHECK(run_psweep(vu, vz, 0, XC, nullptr, nullptr, Lst, nullptr, l.ioffL, s, err));
+    T3F_CHECK(run_psweep(vv, vz, 1, XC + xslices_size(vu), nullptr, nullptr, Rst, nullptr, l.ioffR, s, err));
     T3F_CHECK(run_passemble(vu, vz, Lst, Rst, l.ioffL, c, part, l.nchunks, s));
     k_reduce_chunks<<<256, 256, 0, s>>>(part, l.nchunks, l.gsize, part);
     T3F_CHECK(launch_status());
@@ -542,18 +540,17 @@ extern "C" t3f_status t3f_project_sum_backward(const t3f_tt* U, const t3f_tt* V,
     const float* Vp = static_cast<const float*>(vv.p);
     int* err = static_cast<int*>(ws);
     if (cudaMemsetAsync(ws, 0, sizeof(int), s) != cudaSuccess) return T3F_ERR_CUDA;
-    T3F_CHECK(run_psweep(vu, vz, 0, Up, Vp, Wc, Lst, Pst, l.ioffL, s, err));
-    // the right sweep and the gradient kernel stage their slices from transposed copies of
-    // V, U and W (16-byte copies)
-    float* XT = reinterpret_cast<float*>(w + l.offXT);
-    long long toff[T3F_MAX_D];
-    const long long tsz = xtranspose_offsets(vu, toff);
-    const float* srcs[3] = {Vp, Up, Wc};
-    T3F_CHECK(run_xtranspose(vu, srcs, 3, XT, s));
-    const float *VT = XT, *UT = XT + tsz, *WT = XT + 2 * tsz;
-    T3F_CHECK(run_psweep(vu, vz, 1, VT, UT, WT, Rst, Qst, l.ioffL, s, err, toff));
-    return run_pgrad(vu, vz, UT, VT, WT, Lst, Rst, Pst, Qst, l.ioffL, c, dZ ? static_cast<float*>(vdz.p) : nullptr,
-                     dc, s, toff);
+    // the sweeps and the gradient kernel bring their slices in by bulk copies of slice-major
+    // copies of U, V, W: left orientation, then right
+    float* XC = reinterpret_cast<float*>(w + l.offXT);
+    const long long tsz = xslices_size(vu);
+    const float* srcs[6] = {Up, Vp, Wc, Up, Vp, Wc};
+    T3F_CHECK(run_xslices(vu, srcs, 0x38u, 6, XC, s));
+    T3F_CHECK(run_psweep(vu, vz, 0, XC, XC + tsz, XC + 2 * tsz, Lst, Pst, l.ioffL, s, err));
+    const float *UR = XC + 3 * tsz, *VR = XC + 4 * tsz, *WR = XC + 5 * tsz;
+    T3F_CHECK(run_psweep(vu, vz, 1, VR, UR, WR, Rst, Qst, l.ioffL, s, err));
+    return run_pgrad(vu, vz, UR, VR, WR, Lst, Rst, Pst, Qst, l.ioffL, c, dZ ? static_cast<float*>(vdz.p) : nullptr,
+                     dc, err, s);
   }
   T3F_CHECK(run_pair_sweep(vu, vz, 0, nullptr, Lst, l.ioffL, s));
   T3F_CHECK(run_pair_sweep(vv, vz, 1, nullptr, Rst, l.ioffR, s));
