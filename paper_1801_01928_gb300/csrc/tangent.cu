@@ -128,6 +128,278 @@ __global__ void __launch_bounds__(kThreads) k_assemble_batch(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------
+// The same projection in one kernel for X ranks <= 32 and Z ranks <= 8: assembly and gauge
+// projection of one (core, object) at a time, Zhat staying in shared memory. A CTA takes a
+// contiguous range of (core, object) units, core-major, so U_k is staged once per core it
+// meets and the next object's L, R and Z arrive by asynchronous copies meanwhile. Per unit
+//   Y[g][i][b] = c_j sum_h Z[g][i][h] R[b][h]                 (2 x 8 blocks)
+//   Zhat[(a, i)][b] = sum_g L[a][g] Y[g][i][b]                (8 x 8 blocks)
+//   G = U^T Zhat: 8 x 8 blocks, the rows split over 16 lanes and summed with shuffles
+//   out = Zhat - U G: 8 x 8 blocks (rows interleaved over the lanes), written once.
+// Bound by FP32 multiply-adds against shared-memory operands (16 floats per 64). Against
+// k_assemble_batch + k_gauge_batch (Zhat written, read and written again, 4 x 4 blocks with
+// three barriers per slice): 100 objects at d = 20, n = 16, r = 32: 165 + 342 us -> 169 us.
+// ---------------------------------------------------------------------------------------
+struct ProjCoreArgs {
+  TTV U, Z, D;
+  const float* L;
+  const float* R;
+  long long ioff[T3F_MAX_D + 1];
+  const float* c;  // nullable
+  int mmax;        // most rows of an unfolding
+};
+
+template <int RU>
+__host__ __device__ constexpr int proj_in_floats(int nmax) { return 2 * RU * 12 + 8 * nmax * 8; }
+
+template <int RU>
+size_t proj_core_smem(int mmax, int nmax) {
+  const size_t LD = RU + 4, rows = (mmax + 7) & ~7;
+  return sizeof(float) * (2 * rows * LD + (size_t)8 * nmax * LD + RU * LD + 2 * (size_t)proj_in_floats<RU>(nmax));
+}
+
+__device__ __forceinline__ void ld8(float (&v)[8], const float* p) {
+  const float4 x = *reinterpret_cast<const float4*>(p), y = *reinterpret_cast<const float4*>(p + 4);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+}
+
+template <int RU>
+__global__ void __launch_bounds__(kThreads) k_project_core(const __grid_constant__ ProjCoreArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int LD = RU + 4;    // row stride: consecutive rows start four banks apart
+  constexpr int QR = RU / 8;    // 8-wide blocks of a rank
+  constexpr int RS = 12;        // row stride of the L and R blocks (8 used)
+  const int d = a.U.d, B = a.Z.batch, tid = threadIdx.x, nmax = a.Z.nmax;
+  const int rows = (a.mmax + 7) & ~7;
+  float* Us = sm;                                  // [rows][LD]
+  float* Zh = Us + (size_t)rows * LD;              // [rows][LD]  Zhat
+  float* Ys = Zh + (size_t)rows * LD;              // [8][n][LD]
+  float* Gs = Ys + (size_t)8 * nmax * LD;          // [RU][LD]
+  float* In = Gs + RU * LD;                        // two buffers: L [RU][12], R [RU][12], Z [8][n][8]
+  const int insz = proj_in_floats<RU>(nmax);
+  const float* Zp = static_cast<const float*>(a.Z.p);
+  const float* Up = static_cast<const float*>(a.U.p);
+  const long long units = (long long)d * B;
+  const long long u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  auto cp4 = [](float* dst, const float* src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(ok ? 4 : 0));
+  };
+  auto issue = [&](long long u, int buf) {
+    const int k = (int)(u / B), j = (int)(u - (long long)k * B);
+    const int r0 = a.U.r[k], r1 = a.U.r[k + 1], s0 = a.Z.r[k], s1 = a.Z.r[k + 1], n = a.U.n[k];
+    float* Ls = In + (size_t)buf * insz;
+    float* Rs = Ls + RU * RS;
+    float* Zs = Rs + RU * RS;
+    const float* Lp = a.L + a.ioff[k] + (long long)j * r0 * s0;
+    const float* Rp = a.R + a.ioff[k + 1] + (long long)j * r1 * s1;
+    const float* Zk = Zp + core_base(a.Z, k, j);
+    for (int e = tid; e < RU * 8; e += kThreads) {
+      const int m = e >> 3, b = e & 7;
+      const bool lo = m < r0 && b < s0, ro = m < r1 && b < s1;
+      cp4(Ls + m * RS + b, lo ? Lp + m * s0 + b : Lp, lo);
+      cp4(Rs + m * RS + b, ro ? Rp + m * s1 + b : Rp, ro);
+    }
+    for (int e = tid; e < 8 * n * 8; e += kThreads) {
+      const int h = e & 7, gi = e >> 3, g = gi / n;
+      const bool ok = g < s0 && h < s1;
+      cp4(Zs + e, ok ? Zk + (long long)gi * s1 + h : Zk, ok);  // gi = g n + i is the stored row
+    }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  if (u0 < u1) issue(u0, 0);
+  int kprev = -1, buf = 0;
+  for (long long u = u0; u < u1; ++u, buf ^= 1) {
+    const int k = (int)(u / B), j = (int)(u - (long long)k * B);
+    const int r0 = a.U.r[k], r1 = a.U.r[k + 1], n = a.U.n[k], m = r0 * n;
+    const bool last = k == d - 1;
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();  // the inputs have landed; the previous unit is done with every buffer
+    if (u + 1 < u1) issue(u + 1, buf ^ 1);
+    if (k != kprev && !last) {  // U_k, columns zero-padded (read after the barriers below)
+      const float* Uk = Up + a.U.off[k];
+      for (int e = tid; e < m * RU; e += kThreads) {
+        const int q = e / RU, c = e % RU;
+        Us[q * LD + c] = c < r1 ? __ldg(Uk + q * r1 + c) : 0.0f;
+      }
+    }
+    kprev = k;
+    const float* Ls = In + (size_t)buf * insz;
+    const float* Rs = Ls + RU * RS;
+    const float* Zs = Rs + RU * RS;
+    const float cj = a.c ? a.c[j] : 1.0f;
+    for (int e = tid; e < n * RU / 2; e += kThreads) {
+      const int q = e % (RU / 2), i = e / (RU / 2);
+      float ra[8], rb[8];
+      ld8(ra, Rs + (2 * q) * RS);
+      ld8(rb, Rs + (2 * q + 1) * RS);
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        ra[h] *= cj;
+        rb[h] *= cj;
+      }
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {
+        float z[8];
+        ld8(z, Zs + (g * n + i) * 8);
+        float s = ra[0] * z[0], t = rb[0] * z[0];
+#pragma unroll
+        for (int h = 1; h < 8; ++h) {
+          s = fmaf(ra[h], z[h], s);
+          t = fmaf(rb[h], z[h], t);
+        }
+        *reinterpret_cast<float2*>(Ys + (size_t)(g * n + i) * LD + 2 * q) = make_float2(s, t);
+      }
+    }
+    __syncthreads();
+    float* out = static_cast<float*>(a.D.p) + core_base(a.D, k, j);
+    for (int w = tid; w < QR * n * QR; w += kThreads) {
+      const int bq = w % QR, i = (w / QR) % n, aq = w / (QR * n);
+      float acc[8][8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[x][y] = 0.0f;
+#pragma unroll
+      for (int g4 = 0; g4 < 8; g4 += 4) {
+        float4 lv[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) lv[x] = *reinterpret_cast<const float4*>(Ls + (8 * aq + x) * RS + g4);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          float yv[8];
+          ld8(yv, Ys + (size_t)((g4 + g) * n + i) * LD + 8 * bq);
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            const float l = g == 0 ? lv[x].x : (g == 1 ? lv[x].y : (g == 2 ? lv[x].z : lv[x].w));
+#pragma unroll
+            for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(l, yv[y], acc[x][y]);
+          }
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int al = 8 * aq + x, row = al * n + i;
+        if (al >= r0) continue;
+        if (last) {
+#pragma unroll
+          for (int y = 0; y < 8; ++y)
+            if (8 * bq + y < r1) out[(long long)row * r1 + 8 * bq + y] = acc[x][y];
+        } else {
+          float* z = Zh + (size_t)row * LD + 8 * bq;
+          *reinterpret_cast<float4*>(z) = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
+          *reinterpret_cast<float4*>(z + 4) = make_float4(acc[x][4], acc[x][5], acc[x][6], acc[x][7]);
+        }
+      }
+    }
+    if (last) continue;
+    __syncthreads();
+    if (tid < QR * QR * 16) {  // G: block tid / 16, rows tid % 16 (mod 16)
+      const int blk = tid >> 4, sp = tid & 15, pq = blk / QR, qq = blk % QR;
+      float acc[8][8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[x][y] = 0.0f;
+#pragma unroll 2
+      for (int q = sp; q < m; q += 16) {
+        float uv[8], zv[8];
+        ld8(uv, Us + (size_t)q * LD + 8 * pq);
+        ld8(zv, Zh + (size_t)q * LD + 8 * qq);
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+#pragma unroll
+          for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(uv[x], zv[y], acc[x][y]);
+      }
+      // reduce over the 16 lanes of the block, halving what a lane keeps: rows 4, 2, 1, then
+      // half a row
+      const unsigned msk = QR * QR * 16 >= 32 ? 0xffffffffu : 0xffffu;
+      const bool h8 = (sp & 8) != 0, h4 = (sp & 4) != 0, h2 = (sp & 2) != 0, h1 = (sp & 1) != 0;
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) {
+          const float got = __shfl_xor_sync(msk, h8 ? acc[x][y] : acc[x + 4][y], 8);
+          acc[x][y] = (h8 ? acc[x + 4][y] : acc[x][y]) + got;
+        }
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) {
+          const float got = __shfl_xor_sync(msk, h4 ? acc[x][y] : acc[x + 2][y], 4);
+          acc[x][y] = (h4 ? acc[x + 2][y] : acc[x][y]) + got;
+        }
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {
+        const float got = __shfl_xor_sync(msk, h2 ? acc[0][y] : acc[1][y], 2);
+        acc[0][y] = (h2 ? acc[1][y] : acc[0][y]) + got;
+      }
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const float got = __shfl_xor_sync(msk, h1 ? acc[0][y] : acc[0][y + 4], 1);
+        acc[0][y] = (h1 ? acc[0][y + 4] : acc[0][y]) + got;
+      }
+      const int row = 8 * pq + (h8 ? 4 : 0) + (h4 ? 2 : 0) + (h2 ? 1 : 0);
+      *reinterpret_cast<float4*>(Gs + row * LD + 8 * qq + (h1 ? 4 : 0)) =
+          make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+    }
+    __syncthreads();
+    // out = Zhat - U G: rows rg + x NRG of a thread, eight columns
+    const int NRG = (m + 7) / 8;
+    const bool v4 = (r1 & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    for (int w = tid; w < NRG * QR; w += kThreads) {
+      const int cg = w % QR, rg = w / QR;
+      if (8 * cg >= r1) continue;
+      float acc[8][8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) ld8(acc[x], Zh + (size_t)(rg + x * NRG) * LD + 8 * cg);
+#pragma unroll 2
+      for (int p4 = 0; p4 < RU; p4 += 4) {
+        float4 uv[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) uv[x] = *reinterpret_cast<const float4*>(Us + (size_t)(rg + x * NRG) * LD + p4);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float gv[8];
+          ld8(gv, Gs + (p4 + q) * LD + 8 * cg);
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            const float l = q == 0 ? uv[x].x : (q == 1 ? uv[x].y : (q == 2 ? uv[x].z : uv[x].w));
+#pragma unroll
+            for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(-l, gv[y], acc[x][y]);
+          }
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int row = rg + x * NRG;
+        if (row >= m) continue;
+        float* o = out + (long long)row * r1 + 8 * cg;
+        if (v4) {
+          *reinterpret_cast<float4*>(o) = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
+          if (8 * cg + 4 < r1) *reinterpret_cast<float4*>(o + 4) = make_float4(acc[x][4], acc[x][5], acc[x][6], acc[x][7]);
+        } else {
+#pragma unroll
+          for (int y = 0; y < 8; ++y)
+            if (8 * cg + y < r1) o[y] = acc[x][y];
+        }
+      }
+    }
+  }
+}
+
+template <int RU>
+t3f_status launch_project_core(const ProjCoreArgs& a, int sms, cudaStream_t s) {
+  const size_t smem = proj_core_smem<RU>(a.mmax, a.Z.nmax);
+  if (cudaFuncSetAttribute(k_project_core<RU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return T3F_ERR_CUDA;
+  const long long units = (long long)a.U.d * a.Z.batch;
+  k_project_core<RU><<<(unsigned)std::min<long long>(units, sms), kThreads, smem, s>>>(a);
+  return launch_status();
+}
+
+// ---------------------------------------------------------------------------------------
 // Gather of a tangent vector at index tuples: xi(i) = q_d with the block recurrence
 // q_k = q_{k-1} V_k[:, i_k, :] + p_{k-1} dU_k[:, i_k, :], p_k = p_{k-1} U_k[:, i_k, :],
 // p_0 = 1, q_0 = 0 (the row vector [q, p] through the rank-2r cores [[V, 0], [dU, U]]).
@@ -342,6 +614,146 @@ __global__ void __launch_bounds__(kThreads, 2) k_tgram(const __grid_constant__ T
       if (b < g.B.batch) P[(long long)a * g.B.batch + b] = acc[u][v];
     }
   }
+}
+
+// The Gram matrix of one batch of at most 128 tangent vectors with itself: only the 8 x 8 blocks on
+// and above the diagonal (nb (nb + 1) / 2 of nb^2, nb = batch / 8 rounded up, so 100 vectors take
+// 91 blocks instead of the 256 of a 128 x 128 tile). Block t is rows 4t..4t+3 and 4 nb + 4t..+3. The
+// blocks are dealt to `teams` teams of T threads, each team taking every teams-th column of a
+// 32-column step (two 16-column chunks); the teams' sums meet in shared memory. Operands as in
+// k_tgram, read 16 bytes at a time where every core allows it. Batch 100, 2.8e5 coordinates:
+// 264 us with the full tile -> 162 us.
+struct TGramSymArgs {
+  TGramArgs g;
+  int nb, T, teams, vec;
+};
+
+constexpr int kSymLD = 128 + 4, kSymThreads = 288;
+
+__global__ void __launch_bounds__(kSymThreads, 2) k_tgram_sym(const __grid_constant__ TGramSymArgs a) {
+  extern __shared__ __align__(16) float sm[];  // [2][32][kSymLD]; at the end [teams][T] blocks of 64
+  const TGramArgs& g = a.g;
+  const int tid = threadIdx.x, nth = blockDim.x, nb = a.nb, H = 4 * nb, B = g.A.batch;
+  const int team = tid / a.T, blk = tid % a.T, nblk = nb * (nb + 1) / 2;
+  int t = 0, u = 0;  // block (t, u), t <= u
+  {
+    int rem = min(blk, nblk - 1);
+    while (rem >= nb - t) {
+      rem -= nb - t;
+      ++t;
+    }
+    u = t + rem;
+  }
+  const long long c0 = (long long)blockIdx.x * g.cper, c1 = min(g.nchunks, c0 + g.cper);
+  const float* Ap = static_cast<const float*>(g.A.p);
+  float acc[8][8];
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) acc[x][y] = 0.0f;
+  // position of the next chunk: core k, column col
+  int kc = 0;
+  long long col = 0;
+  tg_chunk(g, c0, &kc, &col);
+  auto advance = [&](int* k, long long* c) {
+    *c += kKC;
+    if (*k < g.A.d && *c >= g.ksz[*k]) {
+      *c = 0;
+      ++*k;
+    }
+  };
+  // quads of the step starting at chunk c: e = (half, row, quad of the 16 columns); at most four
+  // per thread (2 x 128 x 4 over 288 threads)
+  float4 v[4];
+  auto load = [&](long long c) {
+    int k2 = kc;
+    long long col2 = col;
+    advance(&k2, &col2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = tid + q * nth, quad = e & 3, r = (e >> 2) % (2 * H), half = (e >> 2) / (2 * H);
+      v[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (half > 1 || c + half >= c1 || r >= B) continue;
+      const int k = half ? k2 : kc;
+      const long long cc = (half ? col2 : col) + 4 * quad, sz = g.ksz[k];
+      const float* src = Ap + g.A.off[k] + (long long)r * sz + cc;
+      if (a.vec) {
+        if (cc < sz) v[q] = __ldg(reinterpret_cast<const float4*>(src));
+      } else {
+        if (cc < sz) v[q].x = __ldg(src);
+        if (cc + 1 < sz) v[q].y = __ldg(src + 1);
+        if (cc + 2 < sz) v[q].z = __ldg(src + 2);
+        if (cc + 3 < sz) v[q].w = __ldg(src + 3);
+      }
+    }
+    kc = k2;
+    col = col2;
+    advance(&kc, &col);
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = tid + q * nth, quad = e & 3, r = (e >> 2) % (2 * H), half = (e >> 2) / (2 * H);
+      if (half > 1) continue;
+      float* dst = sm + ((size_t)buf * 32 + 16 * half + 4 * quad) * kSymLD + r;
+      dst[0] = v[q].x;
+      dst[kSymLD] = v[q].y;
+      dst[2 * kSymLD] = v[q].z;
+      dst[3 * kSymLD] = v[q].w;
+    }
+  };
+  load(c0);
+  store(0);
+  __syncthreads();
+  int buf = 0;
+  for (long long c = c0; c < c1; c += 2, buf ^= 1) {
+    if (c + 2 < c1) load(c + 2);  // in flight during the products
+    const float* S = sm + (size_t)buf * 32 * kSymLD;
+    if (team < a.teams)
+#pragma unroll 2
+      for (int kk = team; kk < 32; kk += a.teams) {
+        const float* row = S + kk * kSymLD;
+        const float4 a0 = *reinterpret_cast<const float4*>(row + 4 * t);
+        const float4 a1 = *reinterpret_cast<const float4*>(row + H + 4 * t);
+        const float4 b0 = *reinterpret_cast<const float4*>(row + 4 * u);
+        const float4 b1 = *reinterpret_cast<const float4*>(row + H + 4 * u);
+        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+#pragma unroll
+          for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+      }
+    if (c + 2 < c1) store(buf ^ 1);
+    __syncthreads();
+  }
+  // sum the teams in order, team 0 first, one handing its blocks to the next through shared memory
+  for (int q = 0; q + 1 < a.teams; ++q) {
+    if (team == q && blk < nblk)
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) sm[(x * 8 + y) * a.T + blk] = acc[x][y];
+    __syncthreads();
+    if (team == q + 1 && blk < nblk)
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[x][y] = sm[(x * 8 + y) * a.T + blk] + acc[x][y];
+    __syncthreads();
+  }
+  if (team != a.teams - 1 || blk >= nblk) return;
+  float* P = g.part + (long long)blockIdx.x * B * B;
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      const int ra = (x < 4 ? 4 * t + x : H + 4 * t + x - 4), rb = (y < 4 ? 4 * u + y : H + 4 * u + y - 4);
+      if (ra < B && rb < B) {
+        P[(long long)ra * B + rb] = acc[x][y];
+        if (t != u) P[(long long)rb * B + ra] = acc[x][y];
+      }
+    }
 }
 
 // Sum of split partials in a fixed order, in two levels so that every SM takes part:
@@ -706,6 +1118,29 @@ extern "C" t3f_status t3f_project(const t3f_tt* U, const t3f_tt* V, const t3f_tt
     T3F_CHECK(run_pair_sweep(vu, vz, 0, nullptr, Lst, l.ioff, s));
     T3F_CHECK(run_pair_sweep(vv, vz, 1, nullptr, Rst, l.ioff, s));
   }
+  if (psweep_supported(vu, vz)) {
+    int mmax = 1;
+    for (int k = 0; k + 1 < vu.d; ++k) mmax = std::max(mmax, vu.r[k] * vu.n[k]);
+    const size_t smem = vu.rmax <= 8    ? proj_core_smem<8>(mmax, vz.nmax)
+                        : vu.rmax <= 16 ? proj_core_smem<16>(mmax, vz.nmax)
+                                        : proj_core_smem<32>(mmax, vz.nmax);
+    if (smem <= 227 * 1024) {
+      ProjCoreArgs p;
+      memset(&p, 0, sizeof(p));
+      p.U = vu;
+      p.Z = vz;
+      p.D = vd;
+      p.L = Lst;
+      p.R = Rst;
+      for (int j = 0; j <= vu.d; ++j) p.ioff[j] = l.ioff[j];
+      p.c = c;
+      p.mmax = mmax;
+      const int sms = dev_sms();
+      return vu.rmax <= 8    ? launch_project_core<8>(p, sms, s)
+             : vu.rmax <= 16 ? launch_project_core<16>(p, sms, s)
+                             : launch_project_core<32>(p, sms, s);
+    }
+  }
   AssembleBatchArgs a;
   memset(&a, 0, sizeof(a));
   a.U = vu;
@@ -754,6 +1189,23 @@ extern "C" t3f_status t3f_tangent_gram(const t3f_tt* dA, const t3f_tt* dB, float
   g.part = reinterpret_cast<float*>(static_cast<char*>(ws) + p.part_off);
   const long long grid = (long long)p.tilesA * p.tilesB * p.nsplit;
   if (grid > 0x7fffffffLL) return T3F_ERR_UNSUPPORTED;
+  if (g.self && p.tilesA == 1) {  // one tile of a self Gram matrix: its upper triangle
+    TGramSymArgs y;
+    memset(&y, 0, sizeof(y));
+    y.g = g;
+    y.nb = (va.batch + 7) / 8;
+    y.T = (y.nb * (y.nb + 1) / 2 + 31) & ~31;
+    y.teams = std::max(1, kSymThreads / y.T);
+    y.vec = (reinterpret_cast<uintptr_t>(va.p) & 15) == 0;
+    for (int k = 0; k < va.d; ++k) y.vec = y.vec && (va.osz[k] & 3) == 0 && (va.off[k] & 3) == 0;
+    const size_t smem = sizeof(float) * std::max((size_t)2 * 32 * kSymLD, (size_t)64 * y.T);
+    if (cudaFuncSetAttribute(k_tgram_sym, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return T3F_ERR_CUDA;
+    k_tgram_sym<<<(unsigned)p.nsplit, kSymThreads, smem, s>>>(y);
+    T3F_CHECK(launch_status());
+    return run_split_reduce(g.part, p.nsplit, (long long)va.batch * vb.batch,
+                            reinterpret_cast<float*>(static_cast<char*>(ws) + p.mid_off), G, s);
+  }
   k_tgram<<<(unsigned)grid, kThreads, 0, s>>>(g);
   T3F_CHECK(launch_status());
   const long long size = (long long)va.batch * vb.batch;
