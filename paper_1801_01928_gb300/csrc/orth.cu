@@ -15,8 +15,19 @@
 // partial sums per CTA (x.x and x.W[:, l] below the diagonal, plus row j), exchanged through
 // distributed shared memory behind a single cluster barrier per column (the publish slots
 // alternate between two buffers). R is then broadcast to every CTA and Q = W R^{-1} is
-// recovered row by row by a triangular solve that needs no further communication. The
-// working cores keep their original row strides so every in-place update touches only the
+// recovered row by row by a triangular solve that needs no further communication.
+//
+// Tall unfoldings of at most 32 columns first try a factorisation with two exchanges instead of
+// one per column (cqr_step): a Cholesky factor R1 of the Gram matrix taken in FP32 preconditions
+// W, Q1 = W R1^{-1} in FP64 is orthonormal to some 1e-6, and one FP64 Gram matrix of Q1 corrects
+// both factors to FP64 accuracy. The departure of Q1 from orthonormality is measured; where it
+// is not small (ill-conditioned or nearly square unfoldings) the Householder columns run. X of
+// config 5 (d = 20, n = 16, r = 32, 57 factorisations): 6.80 ms with Householder columns alone (3.3
+// us each: one cluster barrier, four block barriers and the FP64 chain of the reflector), 2.53 ms
+// now, 40 us a factorisation, of which the 2.3 thousand FP64 warp instructions of a CTA's 32 rows
+// at some 16 clocks each are 18 us.
+//
+// The working cores keep their original row strides so every in-place update touches only the
 // rows or columns its CTA owns.
 #include <cooperative_groups.h>
 #include <math.h>
@@ -65,29 +76,334 @@ __device__ __forceinline__ long long w_addr(int lr, int q, int l, const Dims& dm
   return ((long long)l * dm.n + i) * R1 + b;
 }
 
-// One QR step of a sweep on core k (updates dims for core k and its neighbour).
-__device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int lr,
-                        const OrthSmem& s, cg::cluster_group& cluster) {
-  const int P = a.P;
-  const int rank = (int)cluster.block_rank();
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const Dims dm = dims[k];
-  const int m = lr ? dm.r0 * dm.n : dm.n * dm.r1;
-  const int c = lr ? dm.r1 : dm.r0;
-  const int kk = m < c ? m : c;
-  const int rp = (m + P - 1) / P;
-  const int row0 = rank * rp;
-  const int nrow = max(0, min(m, row0 + rp) - row0);
-  double* core = base + a.coff[k];
-  const int R1 = a.R1[k];
+// Entry e of a packed upper triangle, column by column: row p <= column q.
+__device__ __forceinline__ void tri_pq(int e, int* p, int* q) {
+  int c = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+  while (c * (c + 1) / 2 > e) --c;
+  while ((c + 1) * (c + 2) / 2 <= e) ++c;
+  *q = c;
+  *p = e - c * (c + 1) / 2;
+}
 
-  cluster.sync();  // previous step's global writes are visible; remote smem reads are done
-  for (int e = tid; e < nrow * c; e += nth) {
-    const int q = e / c, l = e % c;
-    s.W[e] = core[w_addr(lr, row0 + q, l, dm, R1)];
+// The same triangle of order c row by row (p = c - 1 first), and by diagonals q - p (longest first):
+// the lanes of a warp then run sums of nearly equal length.
+__device__ __forceinline__ void tri_row(int e, int c, int* p, int* q) {
+  int a, b;
+  tri_pq(e, &a, &b);
+  *p = c - 1 - b;
+  *q = *p + a;
+}
+__device__ __forceinline__ void tri_diag(int e, int c, int* p, int* q) {
+  int a, b;
+  tri_pq(e, &a, &b);
+  *p = a;
+  *q = a + c - 1 - b;
+}
+
+constexpr int kCqrMax = 32;            // columns
+constexpr int kCqrLd = kCqrMax + 1;
+constexpr int kCqrTri = kCqrMax * (kCqrMax + 1) / 2;
+constexpr int kCqrPer = (kCqrTri + kOrthThreads - 1) / kOrthThreads;  // triangle entries per thread
+
+// U <- phi(E - U^T U), `its` times from U = phi(E) (phi: strict upper part plus half the
+// diagonal), so that (I + U)^T (I + U) = I + E up to |E|^(its + 2); then C <- U - U C from C = U,
+// so that (I + U)(I - C) = I to the same order. The second-order products run in T on Ub / Cb, the
+// leading terms in FP64 (e: this thread's entries of E, by rows; results in Um and Cm).
+template <typename T>
+__device__ void cqr_series(const double* e, int c, int its, T* Ub, T* Cb, double* Um, double* Cm) {
+  const int tid = threadIdx.x, nt = c * (c + 1) / 2;
+  int p[kCqrPer], q[kCqrPer];
+#pragma unroll
+  for (int x = 0; x < kCqrPer; ++x) {
+    const int en = tid + x * kOrthThreads;
+    p[x] = 0;
+    q[x] = -1;
+    if (en < nt) {
+      tri_row(en, c, &p[x], &q[x]);
+      Ub[p[x] * kCqrLd + q[x]] = (T)(p[x] == q[x] ? 0.5 * e[x] : e[x]);
+    }
   }
   __syncthreads();
+  for (int it = 0; it < its; ++it) {
+    T t[kCqrPer];
+#pragma unroll
+    for (int x = 0; x < kCqrPer; ++x) {
+      t[x] = (T)0;
+      if (q[x] >= 0)
+#pragma unroll 8
+        for (int r = 0; r <= p[x]; ++r) t[x] += Ub[r * kCqrLd + p[x]] * Ub[r * kCqrLd + q[x]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < kCqrPer; ++x)
+      if (q[x] >= 0) {
+        const double v = e[x] - (double)t[x], u = p[x] == q[x] ? 0.5 * v : v;
+        Ub[p[x] * kCqrLd + q[x]] = (T)u;
+        if (it == its - 1) {
+          Um[p[x] * kCqrLd + q[x]] = u;
+          Cb[p[x] * kCqrLd + q[x]] = (T)u;
+        }
+      }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int x = 0; x < kCqrPer; ++x)
+    if (q[x] >= 0) tri_diag(tid + x * kOrthThreads, c, &p[x], &q[x]);
+  for (int it = 0; it < its; ++it) {
+    T t[kCqrPer];
+#pragma unroll
+    for (int x = 0; x < kCqrPer; ++x) {
+      t[x] = (T)0;
+      if (q[x] >= 0)
+#pragma unroll 8
+        for (int r = p[x]; r <= q[x]; ++r) t[x] += Ub[p[x] * kCqrLd + r] * Cb[r * kCqrLd + q[x]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < kCqrPer; ++x)
+      if (q[x] >= 0) {
+        const double u = Um[p[x] * kCqrLd + q[x]] - (double)t[x];
+        Cb[p[x] * kCqrLd + q[x]] = (T)u;
+        if (it == its - 1) Cm[p[x] * kCqrLd + q[x]] = u;
+      }
+    __syncthreads();
+  }
+}
 
+// Rows x (8 lanes a row, lane g keeps the columns l = g mod 8 in registers) <- x U^{-1}, U unit upper
+// triangular with row stride T3F_MAX_RANK, then column l times scale[l].
+__device__ __forceinline__ void unit_solve_rows(double* W, int nrow, int c, const double* U, const double* scale) {
+  const int tid = threadIdx.x, g = tid % 8, uend = (c + 7) / 8;
+  for (int q0 = 0; q0 < nrow; q0 += kOrthThreads / 8) {
+    const int q = q0 + tid / 8;
+    const bool qv = q < nrow;
+    double* qr = W + (qv ? q : 0) * c;
+    double x[kCqrMax / 8];
+#pragma unroll
+    for (int u = 0; u < kCqrMax / 8; ++u) {
+      const int l = g + 8 * u;
+      x[u] = (qv && l < c) ? qr[l] : 0.0;
+    }
+#pragma unroll
+    for (int UB = 0; UB < kCqrMax / 8; ++UB) {
+      if (UB >= uend) break;
+      for (int ob = 0; ob < 8; ++ob) {
+        const int b = 8 * UB + ob;
+        if (b >= c) break;
+        const double xb = __shfl_sync(0xffffffffu, x[UB], ob, 8);
+        const double* rb = U + b * T3F_MAX_RANK;
+#pragma unroll
+        for (int u = UB; u < kCqrMax / 8; ++u) {
+          const int l = g + 8 * u;
+          if (u < uend && l > b && l < c) x[u] = fma(-xb, rb[l], x[u]);
+        }
+      }
+    }
+    if (qv)
+#pragma unroll
+      for (int u = 0; u < kCqrMax / 8; ++u) {
+        const int l = g + 8 * u;
+        if (l < c) qr[l] = x[u] * scale[l];
+      }
+  }
+}
+
+// QR of the cluster's m x c unfolding (c <= 32, m >= c), this CTA's rows in s.W (row-major, ld c):
+// on success s.W holds the rows of Q, s.Rs the factor R (diag(R) > 0), and true is returned in every
+// CTA; false (in every CTA: they decide on the same sums) where W is too ill-conditioned for it,
+// with s.W overwritten.
+//   G = W^T W and G = U1^T D^2 U1 in FP32, R1 = D U1 (exact in FP64);  Q1 = W R1^{-1} in FP64;
+//   E = Q1^T Q1 - I in FP64;  (I + U)^T (I + U) = I + E;  Q = Q1 (I + U)^{-1}, R = (I + U) R1.
+// With |E| <= 3e-5 the terms of second order and up are below 1e-9 and FP32 holds them to 1e-16;
+// up to 1e-2 they run in FP64; the series is cut where |E|^(its + 2) < 1e-17.
+__device__ bool cqr_step(const OrthArgs& a, const OrthSmem& s, int nrow, int c, cg::cluster_group& cluster) {
+  const int P = a.P, tid = threadIdx.x, lane = tid & 31, nt = c * (c + 1) / 2;
+  // the second half of the W region is free (c <= 32 of T3F_MAX_RANK = 64 columns)
+  float* Wf = reinterpret_cast<float*>(s.W + (size_t)a.rows_per * kCqrMax);  // rows x c
+  float* pubf = Wf + (size_t)a.rows_per * kCqrMax;                           // triangle
+  double* pubd = reinterpret_cast<double*>(pubf + kCqrTri + (kCqrTri & 1));  // triangle
+  double* sumd = pubd + kCqrTri;                                             // a P-th of it, summed
+  double* Um = sumd + (kCqrTri + 7) / 8;
+  double* Cm = Um + kCqrMax * kCqrLd;
+  float* Uf = reinterpret_cast<float*>(Cm + kCqrMax * kCqrLd);
+  float* Cf = Uf + kCqrMax * kCqrLd;
+  __shared__ float red[kOrthThreads / 32];
+  __shared__ int bad;
+  for (int e = tid; e < nrow * c; e += kOrthThreads) Wf[e] = (float)s.W[e];
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  for (int e = tid; e < nt; e += kOrthThreads) {
+    int p, q;
+    tri_pq(e, &p, &q);
+    float v = 0.0f, w = 0.0f;  // two chains: half the accumulated rounding and latency
+    int r = 0;
+    for (; r + 1 < nrow; r += 2) {
+      v = fmaf(Wf[r * c + p], Wf[r * c + q], v);
+      w = fmaf(Wf[(r + 1) * c + p], Wf[(r + 1) * c + q], w);
+    }
+    if (r < nrow) v = fmaf(Wf[r * c + p], Wf[r * c + q], v);
+    pubf[e] = v + w;
+  }
+  cluster.sync();
+  for (int e = tid; e < nt; e += kOrthThreads) {
+    int p, q;
+    tri_pq(e, &p, &q);
+    float v[16], t = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = r < P ? cluster.map_shared_rank(pubf, r)[e] : 0.0f;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)  // pairwise: the least rounding
+#pragma unroll
+      for (int r = 0; r < o; ++r) v[r] += v[r + o];
+    t = v[0];
+    Uf[p * kCqrLd + q] = t;
+    Uf[q * kCqrLd + p] = t;
+  }
+  __syncthreads();
+  // G = U1^T D^2 U1: warp 0, lane = column
+  if (tid < 32) {
+    float g[kCqrMax];
+#pragma unroll
+    for (int p = 0; p < kCqrMax; ++p) g[p] = p < c && lane < c ? Uf[p * kCqrLd + lane] : 0.0f;
+    bool ok = true;
+    float dj = 1.0f;  // this lane's pivot
+#pragma unroll
+    for (int j = 0; j < kCqrMax; ++j)
+      if (j < c) {
+        const float piv = __shfl_sync(0xffffffffu, g[j], j);
+        ok = ok && piv > 0.0f && piv < 3.0e38f;
+        const float gj = g[j], u = lane == j ? 1.0f : gj * __fdividef(1.0f, piv);
+        if (lane >= j) Uf[j * kCqrLd + lane] = u;
+        dj = lane == j ? piv : dj;
+#pragma unroll
+        for (int p = j + 1; p < kCqrMax; ++p) g[p] = fmaf(-__shfl_sync(0xffffffffu, u, p), gj, g[p]);
+      }
+    if (lane < c) {
+      s.wj[lane] = (double)sqrtf(dj);
+      s.rinv[lane] = 1.0 / s.wj[lane];
+    }
+    if (!ok && lane == 0) bad = 1;
+  }
+  __syncthreads();
+  if (bad) return false;
+  for (int e = tid; e < c * c; e += kOrthThreads) {
+    const int p = e / c, q = e % c;
+    if (q >= p) s.Rs[p * T3F_MAX_RANK + q] = (double)Uf[p * kCqrLd + q];
+  }
+  __syncthreads();
+  unit_solve_rows(s.W, nrow, c, s.Rs, s.rinv);  // Q1 = W U1^{-1} D^{-1}
+  __syncthreads();
+  for (int e = tid; e < nt; e += kOrthThreads) {  // R1 = D U1 (exact: a product of two FP32 values)
+    int p, q;
+    tri_pq(e, &p, &q);
+    s.Rs[p * T3F_MAX_RANK + q] *= s.wj[p];
+  }
+  for (int e = tid; e < nt; e += kOrthThreads) {
+    int p, q;
+    tri_pq(e, &p, &q);
+    double v = 0.0;
+    for (int r = 0; r < nrow; ++r) v = fma(s.W[r * c + p], s.W[r * c + q], v);
+    pubd[e] = v;
+  }
+  cluster.sync();
+  // E: CTA r sums the cluster's entries r npc .. (r + 1) npc - 1, sixteen lanes an entry, and every
+  // CTA then gathers the sums (sixteen remote reads and FP64 additions per entry and CTA otherwise)
+  const int npc = (nt + P - 1) / P, e0 = (int)cluster.block_rank() * npc, e1 = min(nt, e0 + npc);
+  for (int w0 = 0; w0 < 16 * npc; w0 += kOrthThreads) {
+    const int e = e0 + (w0 + tid) / 16, r = tid % 16;
+    double v = e < e1 && r < P ? cluster.map_shared_rank(pubd, r)[e] : 0.0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (r == 0 && e < e1) sumd[e - e0] = v;
+  }
+  cluster.sync();
+  double ev[kCqrPer];
+  float nrm = 0.0f;
+#pragma unroll
+  for (int x = 0; x < kCqrPer; ++x) {
+    const int en = tid + x * kOrthThreads;
+    ev[x] = 0.0;
+    if (en >= nt) continue;
+    int p, q;
+    tri_row(en, c, &p, &q);
+    const int e = q * (q + 1) / 2 + p;
+    const double v = cluster.map_shared_rank(sumd, e / npc)[e % npc];
+    ev[x] = p == q ? v - 1.0 : v;
+    const float f = (float)ev[x];
+    nrm += (p == q ? 1.0f : 2.0f) * f * f;
+  }
+  for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+  if (lane == 0) red[tid >> 5] = nrm;
+  __syncthreads();
+  nrm = 0.0f;
+  for (int w = 0; w < kOrthThreads / 32; ++w) nrm += red[w];
+  nrm = sqrtf(nrm);  // |E| in the Frobenius norm, the same bits in every CTA
+  if (!(nrm < 1e-2f)) return false;
+  if (nrm < 3e-5f) cqr_series<float>(ev, c, nrm < 2e-6f ? 1 : 2, Uf, Cf, Um, Cm);
+  else cqr_series<double>(ev, c, nrm < 1e-4f ? 3 : (nrm < 1e-3f ? 4 : 7), Um, Cm, Um, Cm);
+  // R = (I + U) R1
+  double rv[kCqrPer];
+#pragma unroll
+  for (int x = 0; x < kCqrPer; ++x) {
+    const int e = tid + x * kOrthThreads;
+    if (e >= nt) continue;
+    int p, q;
+    tri_diag(e, c, &p, &q);
+    double v = s.Rs[p * T3F_MAX_RANK + q];
+#pragma unroll 4
+    for (int r = p; r <= q; ++r) v = fma(Um[p * kCqrLd + r], s.Rs[r * T3F_MAX_RANK + q], v);
+    rv[x] = v;
+  }
+  // Q = Q1 - Q1 C: sixteen lanes a row, lane l takes the columns l and c2 - 1 - l (c2 = c rounded up
+  // to even), c2 + 1 steps for every lane
+  const int half = (c + 1) / 2, c2 = 2 * half;
+  for (int r0 = 0; r0 < nrow; r0 += kOrthThreads / 16) {
+    const int r = r0 + tid / 16, l = tid % 16;
+    const bool on = r < nrow && l < half;
+    double lo = 0.0, hi = 0.0;
+    const int ch = c2 - 1 - l;
+    const double* w = s.W + (size_t)(on ? r : 0) * c;
+    if (on) {
+      const int cs = min(ch, c - 1);  // (c odd: lane 0 has no second column)
+      double acc = w[l];
+      hi = w[cs];
+      for (int t = 0; t <= c2; ++t) {  // one fused multiply-add per step for every lane
+        const bool sec = t > l;
+        if (t == l + 1) {
+          lo = acc;
+          acc = hi;
+        }
+        const int r = min(sec ? t - l - 1 : t, cs);
+        acc = fma(-w[r], Cm[r * kCqrLd + (sec ? cs : l)], acc);
+      }
+      hi = acc;
+    }
+    __syncwarp();
+    if (on) {
+      s.W[(size_t)r * c + l] = lo;
+      if (ch < c) s.W[(size_t)r * c + ch] = hi;
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < kCqrPer; ++x) {
+    const int e = tid + x * kOrthThreads;
+    if (e >= nt) continue;
+    int p, q;
+    tri_diag(e, c, &p, &q);
+    s.Rs[p * T3F_MAX_RANK + q] = rv[x];
+  }
+  __syncthreads();
+  return true;
+}
+
+// Householder QR of the cluster's m x c unfolding W (this CTA's nrow rows from row0 in s.W): R (kk x c,
+// diag(R) >= 0) in every CTA's s.Rs, the rows of Q in s.W (ld c).
+__device__ void householder_step(const OrthArgs& a, const double* core, const Dims& dm, int R1, int lr, int m, int c,
+                                 int rp, int row0, int nrow, const OrthSmem& s, cg::cluster_group& cluster) {
+  const int P = a.P, tid = threadIdx.x, nth = blockDim.x;
+  const int kk = m < c ? m : c;
   for (int j = 0; j < kk; ++j) {
     const int par = j & 1;
     double* pub = s.pub + par * T3F_MAX_RANK;
@@ -236,6 +552,67 @@ __device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int 
     }
   }
   __syncthreads();
+}
+
+// out(a, x) = sum_{al >= a} R(a, al) in(al, x) for a < kk, x < nx: the lanes of a warp run over x with
+// one row a (sums of equal length), and a thread takes the rows a and kk - 1 - a together, so every
+// thread does the same work on two independent chains.
+template <class FR, class FI, class FO>
+__device__ __forceinline__ void push_rows(int kk, int c, int nx, FR R, FI in, FO out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int na = (kk + 1) / 2, ng = (nx + 31) / 32;
+  for (int w = warp; w < na * ng; w += nw) {
+    const int a = w % na, b = kk - 1 - a, x = (w / na) * 32 + lane;  // a <= b
+    if (x >= nx) continue;
+    double u = 0.0, v = 0.0;
+    int al = a;
+    for (; al < b; ++al) u = fma(R(a, al), in(al, x), u);
+    for (; al < c; ++al) {
+      const double t = in(al, x);
+      u = fma(R(a, al), t, u);
+      v = fma(R(b, al), t, v);
+    }
+    out(a, x, u);
+    if (b != a) out(b, x, v);
+  }
+}
+
+// One QR step of a sweep on core k (updates dims for core k and its neighbour).
+__device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int lr,
+                        const OrthSmem& s, cg::cluster_group& cluster) {
+  const int P = a.P;
+  const int rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const Dims dm = dims[k];
+  const int m = lr ? dm.r0 * dm.n : dm.n * dm.r1;
+  const int c = lr ? dm.r1 : dm.r0;
+  const int kk = m < c ? m : c;
+  const int rp = (m + P - 1) / P;
+  const int row0 = rank * rp;
+  const int nrow = max(0, min(m, row0 + rp) - row0);
+  double* core = base + a.coff[k];
+  const int R1 = a.R1[k];
+
+  cluster.sync();  // previous step's global writes are visible; remote smem reads are done
+  for (int e = tid; e < nrow * c; e += nth) {
+    const int q = e / c, l = e % c;
+    s.W[e] = core[w_addr(lr, row0 + q, l, dm, R1)];
+  }
+  __syncthreads();
+
+  bool done = false;
+  if (c <= kCqrMax && m >= c) {
+    done = cqr_step(a, s, nrow, c, cluster);
+    if (!done) {  // the rows again, for the Householder columns
+      __syncthreads();
+      for (int e = tid; e < nrow * c; e += nth) {
+        const int q = e / c, l = e % c;
+        s.W[e] = core[w_addr(lr, row0 + q, l, dm, R1)];
+      }
+      __syncthreads();
+    }
+  }
+  if (!done) householder_step(a, core, dm, R1, lr, m, c, rp, row0, nrow, s, cluster);
   Dims nd = dm;
   if (lr) nd.r1 = kk; else nd.r0 = kk;
   for (int e = tid; e < nrow * kk; e += nth) {
@@ -257,33 +634,29 @@ __device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int 
       s.W[e] = nb[((long long)al * nx.n + i) * R1n + b];
     }
     __syncthreads();
-    for (int e = tid; e < kk * nc; e += nth) {
-      const int a2 = e / nc, qq = e % nc, q = c0 + qq;
-      const int i = q / nx.r1, b = q % nx.r1;
-      double acc = 0.0;
-      for (int al = a2; al < c; ++al) acc += s.Rs[a2 * T3F_MAX_RANK + al] * s.W[al * nc + qq];
-      nb[((long long)a2 * nx.n + i) * R1n + b] = acc;
-    }
+    push_rows(kk, c, nc, [&](int a2, int al) { return s.Rs[a2 * T3F_MAX_RANK + al]; },
+              [&](int al, int qq) { return s.W[al * nc + qq]; },
+              [&](int a2, int qq, double v) {
+                const int q = c0 + qq, i = q / nx.r1, b = q % nx.r1;
+                nb[((long long)a2 * nx.n + i) * R1n + b] = v;
+              });
   } else {
     const Dims pv = dims[k - 1];  // (r0', n', c)
     double* pb = base + a.coff[k - 1];
     const int R1p = a.R1[k - 1];
     const int rows = pv.r0 * pv.n;
     const int rq = (rows + P - 1) / P, q0 = rank * rq, nq = max(0, min(rows, q0 + rq) - q0);
+    const int ldw = c | 1;  // (rows are read across the lanes)
     for (int e = tid; e < nq * c; e += nth) {
       const int q = e / c, b = e % c;
-      s.W[e] = pb[(long long)(q0 + q) * R1p + b];
+      s.W[q * ldw + b] = pb[(long long)(q0 + q) * R1p + b];
     }
     __syncthreads();
-    for (int e = tid; e < nq * kk; e += nth) {
-      const int q = e / kk, a2 = e % kk;
-      double acc = 0.0;
-      for (int b = a2; b < c; ++b) acc += s.W[q * c + b] * s.Rs[a2 * T3F_MAX_RANK + b];
-      pb[(long long)(q0 + q) * R1p + a2] = acc;
-    }
+    push_rows(kk, c, nq, [&](int a2, int b) { return s.Rs[a2 * T3F_MAX_RANK + b]; },
+              [&](int b, int q) { return s.W[q * ldw + b]; },
+              [&](int a2, int q, double v) { pb[(long long)(q0 + q) * R1p + a2] = v; });
   }
-  __syncthreads();
-  __threadfence();
+  __syncthreads();  // (the cluster barrier that opens the next step publishes the global writes)
   if (tid == 0) {
     if (lr) {
       dims[k].r1 = kk;
