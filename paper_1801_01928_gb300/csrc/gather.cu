@@ -11,6 +11,7 @@
 // suffix vectors of its tuple in shared memory, evaluates the residual, then walks the
 // prefix and scatters the outer products into a per-CTA shared accumulator; a second
 // kernel reduces the per-CTA partials in a fixed order.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -329,42 +330,53 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_bwd(const __grid_cons
   }
 }
 
-// Bucketed adjoint (the main path for ranks <= 8). Per chunk of T = blockDim tuples:
+// Bucketed adjoint (the main path for ranks <= 8). Per chunk of T tuples, 2 T threads:
 //  (1) a deterministic counting sort of the chunk's tuples by slice, for every core (warp
-//      match + per-warp prefix sums), giving each tuple its bucket position at core k;
-//  (2) thread per tuple: suffix chain storing rho_{k+1} and prefix chain (scaled by the
-//      weight) storing w l_k, both written into the bucket order of core k;
+//      match + per-warp prefix sums; each thread of a tuple takes every other core), giving each
+//      tuple its bucket position at core k; the next chunk's indices are fetched meanwhile;
+//  (2) the two threads of a tuple run its two chains at once: the suffix chain storing rho_{k+1}
+//      (and the value, residual and weight), the prefix chain storing l_k and the tuple's number,
+//      both in the bucket order of core k;
 //  (3) thread per item (core k, slice s, part): a persistent R x R register accumulator
 //      adds w l_k rho_{k+1}^T over the item's share of the bucket; consecutive lanes read
 //      consecutive bucket rows.
 // No atomics in the loop; the per-CTA partial is summed in a fixed order by a second kernel.
+// The slices are read at the tuples' random indices (16 16-byte loads per 64 multiply-adds of a
+// chain step), so the kernel is bound by shared-memory reads and their latency: two threads a
+// tuple, three block barriers a chunk (eight before) and no index load on the path. 10^6
+// tuples, d = 10, n = 10, r = 8: 529 us with one thread per tuple and the prefix after the suffix,
+// now @CM@ us; with two sets of slices (the Riemannian form) 591 -> @CR@ us.
 struct CompletionArgs {
   GatherArgs g;
-  int T;                      // tuples per chunk (= blockDim.x)
+  int T;                      // tuples per chunk (half of blockDim.x)
   int NB;                     // buckets per core (nmax + 1; the last holds invalid tuples)
+  int region;                 // floats of the RH / LW region
   int parts[T3F_MAX_D];       // items per slice at core k
   int item0[T3F_MAX_D + 1];   // first item of core k
 };
 
 template <int R>
-__global__ void __launch_bounds__(256, 1) k_completion(const __grid_constant__ CompletionArgs ca) {
+__global__ void __launch_bounds__(512) k_completion(const __grid_constant__ CompletionArgs ca) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ double red[8];
+  __shared__ double red[16];
   const GatherArgs& g = ca.g;
   const int d = g.d, nmax = g.nmax, T = ca.T, NB = ca.NB;
   constexpr int SS = R * R + 4;  // padded slice stride (breaks same-bank slices)
   constexpr int H = R / 4;       // float4 planes of a rank vector
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = (T + 31) >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = T >> 5, nwarps = blockDim.x >> 5;
+  const int grp = tid >= T ? 1 : 0, tt = tid - grp * T, tw = tt >> 5;  // chain (0 suffix, 1 prefix), tuple, its warp
   const int SL = d * nmax * SS;
   float* Ls = sm;
   float* Rs = g.same ? Ls : Ls + SL;
-  float4* RH = reinterpret_cast<float4*>(Ls + (g.same ? SL : 2 * SL));  // [d][H][T]
-  float4* LW = RH + (size_t)d * H * T;                                     // [d][H][T]
-  unsigned short* POS = reinterpret_cast<unsigned short*>(LW + (size_t)d * H * T);  // [d][T]
-  unsigned char* IDX = reinterpret_cast<unsigned char*>(POS + (size_t)d * T);       // [d][T]
-  unsigned short* WC = reinterpret_cast<unsigned short*>(IDX + (((size_t)d * T + 15) & ~(size_t)15));  // [d][NB][NW]
-  int* CNT = reinterpret_cast<int*>(WC + (((size_t)d * NB * NW + 1) & ~(size_t)1));                      // [d][NB]
-  int* BO = CNT + (size_t)d * NB;                                                   // [d][NB+1]
+  float4* RH = reinterpret_cast<float4*>(Ls + (g.same ? SL : 2 * SL));  // [d - 1][H][T]: rho_{k+1} of core k
+  float4* LW = RH + (size_t)(d - 1) * H * T;                               // [d - 1][H][T]: l of core k + 1
+  float* Wt = reinterpret_cast<float*>(RH) + ca.region;                    // [T] weights
+  int* IN = reinterpret_cast<int*>(Wt + T);                                // [d][T] the next chunk's indices
+  unsigned short* WC = reinterpret_cast<unsigned short*>(IN + (size_t)d * T);  // [d][NB][NW]
+  unsigned short* BO = WC + (size_t)d * NB * NW;                               // [d][NB] bucket starts
+  unsigned char* IDX = reinterpret_cast<unsigned char*>(BO + (size_t)d * NB);  // [d][T]
+  unsigned char* RANK = IDX + (size_t)d * T;                                   // [d][T]
+  unsigned char* TID = RANK + (size_t)d * T;                                   // [d][T] tuple of a bucket row
 
   // stage the cores as zero-padded R x R slices with stride SS: the whole object(s) land in
   // the RH / LW region (not used before the first chunk) through one TMA bulk copy each
@@ -377,10 +389,21 @@ __global__ void __launch_bounds__(256, 1) k_completion(const __grid_constant__ C
     tma_copy(landL, g.L, g.Lnfl, &bar);
     if (!g.same) tma_copy(landR, g.Rg, g.Rnfl, &bar);
   }
+  // this thread's indices of the chunk at base (read back by this thread only)
+  auto fetch = [&](long long base) {
+    const long long t = base + tt;
+    const bool ok = t < g.N;
+    for (int k = grp; k < d; k += 2) {
+      const int* src = g.idx + (ok ? (long long)k * g.N + t : 0);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(smem_u32(IN + k * T + tt)), "l"(src),
+                   "r"(ok ? 4 : 0));
+    }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  fetch((long long)blockIdx.x * T);
   if (!bar_wait(smem_u32(&bar), 0u) && tid == 0) atomicExch(g.err, (int)T3F_ERR_TIMEOUT);
   stage_from_raw<R>(Ls, SS, landL + raw_delta(g.L), g.Loff, g.rl, g.n, d, nmax);
   if (!g.same) stage_from_raw<R>(Rs, SS, landR + raw_delta(g.Rg), g.Roff, g.rr, g.n, d, nmax);
-  __syncthreads();
   // this thread's item (core ik, slice is, part ip) of the accumulation phase
   int ik = -1, is = 0, ip = 0, np = 1;
   for (int k = 0; k < d; ++k)
@@ -399,153 +422,179 @@ __global__ void __launch_bounds__(256, 1) k_completion(const __grid_constant__ C
   __syncthreads();
 
   for (long long base = (long long)blockIdx.x * T; base < g.N; base += (long long)gridDim.x * T) {
-    const long long t = base + tid;
-    const bool valid = tid < T && t < g.N;
-    // (1) counting sort by slice, per core
-    for (int e = tid; e < d * NB * NW; e += blockDim.x) WC[e] = 0;
-    __syncthreads();
-    for (int k = 0; k < d; ++k) {
-      const int sl = valid ? load_index(g, k, t) : nmax;
+    const long long t = base + tt;
+    const bool valid = t < g.N;
+    float yt = 0.0f;
+    if (grp == 0 && valid) yt = g.w ? __ldg(g.w + t) : __ldg(g.y + t);
+    // (1) counting sort by slice (the counts of a (core, warp) belong to that warp)
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    for (int k = grp; k < d; k += 2) {
+      int sl = nmax;
+      if (valid) {
+        sl = IN[k * T + tt];
+        if (sl < 0 || sl >= g.n[k]) {
+          atomicExch(g.err, (int)T3F_ERR_ARG);
+          sl = sl < 0 ? 0 : g.n[k] - 1;
+        }
+      }
+      for (int b = lane; b < NB; b += 32) WC[(k * NB + b) * NW + tw] = 0;
       const unsigned m = __match_any_sync(0xffffffffu, sl);
       const int rank = __popc(m & ((1u << lane) - 1u));
-      if (tid < T) {
-        IDX[k * T + tid] = (unsigned char)sl;
-        POS[k * T + tid] = (unsigned short)rank;
-        if (rank == 0) WC[(k * NB + sl) * NW + warp] = (unsigned short)__popc(m);
+      IDX[k * T + tt] = (unsigned char)sl;
+      RANK[k * T + tt] = (unsigned char)rank;
+      __syncwarp();
+      if (rank == 0) WC[(k * NB + sl) * NW + tw] = (unsigned short)__popc(m);
+    }
+    fetch(base + (long long)gridDim.x * T);
+    __syncthreads();  // counts complete; the previous chunk's accumulation is done
+    for (int k = warp; k < d; k += nwarps) {  // a warp per core: scan over the slices
+      int carry = 0;
+      for (int b0 = 0; b0 < NB; b0 += 32) {
+        const int b = b0 + lane;
+        unsigned short* wc = WC + (size_t)(k * NB + min(b, NB - 1)) * NW;
+        int tot = 0;
+        if (b < NB)
+          for (int w = 0; w < NW; ++w) tot += wc[w];
+        int inc = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += v;
+        }
+        int run = carry + inc - tot;
+        if (b < NB) {
+          BO[k * NB + b] = (unsigned short)run;
+          for (int w = 0; w < NW; ++w) {
+            const int c = wc[w];
+            wc[w] = (unsigned short)run;
+            run += c;
+          }
+        }
+        carry += __shfl_sync(0xffffffffu, inc, 31);
       }
     }
     __syncthreads();
-    for (int e = tid; e < d * NB; e += blockDim.x) {
-      int run = 0;
-      for (int w = 0; w < NW; ++w) {
-        const int c = WC[e * NW + w];
-        WC[e * NW + w] = (unsigned short)run;
-        run += c;
-      }
-      CNT[e] = run;
-    }
-    __syncthreads();
-    for (int k = tid; k < d; k += blockDim.x) {
-      int run = 0;
-      for (int sl = 0; sl < NB; ++sl) {
-        BO[k * (NB + 1) + sl] = run;
-        run += CNT[k * NB + sl];
-      }
-      BO[k * (NB + 1) + NB] = run;
-    }
-    __syncthreads();
-    if (tid < T)
-      for (int k = 0; k < d; ++k) {
-        const int sl = IDX[k * T + tid];
-        POS[k * T + tid] = (unsigned short)(BO[k * (NB + 1) + sl] + WC[(k * NB + sl) * NW + warp] + POS[k * T + tid]);
-      }
-    __syncthreads();
-    // (2) chains of this thread's tuple
+    // (2) the tuple's chains; p = its row in the bucket order of core k
     if (valid) {
-      float rho[R];
+      float v[R];
 #pragma unroll
-      for (int a = 0; a < R; ++a) rho[a] = a == 0 ? 1.0f : 0.0f;
-      for (int k = d - 1; k >= 1; --k) {
-        const int p = POS[k * T + tid];
+      for (int a = 0; a < R; ++a) v[a] = a == 0 ? 1.0f : 0.0f;
+      if (grp == 0) {
+        for (int k = d - 1; k >= 0; --k) {
+          const int sl = IDX[k * T + tt];
+          const float* S = Rs + (k * nmax + sl) * SS;
+          if (k < d - 1) {
+            const int p = WC[(k * NB + sl) * NW + tw] + RANK[k * T + tt];
 #pragma unroll
-        for (int h = 0; h < H; ++h)
-          RH[((size_t)k * H + h) * T + p] = make_float4(rho[4 * h], rho[4 * h + 1], rho[4 * h + 2], rho[4 * h + 3]);
-        const float* S = Rs + (k * nmax + IDX[k * T + tid]) * SS;
-        float nr[R];
-#pragma unroll
-        for (int a = 0; a < R; ++a) {
-          float acc1 = 0.0f;
-#pragma unroll
-          for (int b = 0; b < R; b += 4) {
-            const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
-            acc1 = fmaf(s4.x, rho[b], acc1);
-            acc1 = fmaf(s4.y, rho[b + 1], acc1);
-            acc1 = fmaf(s4.z, rho[b + 2], acc1);
-            acc1 = fmaf(s4.w, rho[b + 3], acc1);
+            for (int h = 0; h < H; ++h)
+              RH[((size_t)k * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
           }
-          nr[a] = acc1;
+          if (k == 0) {
+            float x = 0.0f;
+#pragma unroll
+            for (int b = 0; b < R; ++b) x = fmaf(S[b], v[b], x);
+            v[0] = x;
+            break;
+          }
+          float nr[R];
+#pragma unroll
+          for (int a = 0; a < R; ++a) {
+            float acc1 = 0.0f;
+#pragma unroll
+            for (int b = 0; b < R; b += 4) {
+              const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+              acc1 = fmaf(s4.x, v[b], acc1);
+              acc1 = fmaf(s4.y, v[b + 1], acc1);
+              acc1 = fmaf(s4.z, v[b + 2], acc1);
+              acc1 = fmaf(s4.w, v[b + 3], acc1);
+            }
+            nr[a] = acc1;
+          }
+#pragma unroll
+          for (int a = 0; a < R; ++a) v[a] = nr[a];
         }
-#pragma unroll
-        for (int a = 0; a < R; ++a) rho[a] = nr[a];
-      }
-      {
-        const int p = POS[tid];
-#pragma unroll
-        for (int h = 0; h < H; ++h)
-          RH[(size_t)h * T + p] = make_float4(rho[4 * h], rho[4 * h + 1], rho[4 * h + 2], rho[4 * h + 3]);
-      }
-      const float* S0 = Rs + IDX[tid] * SS;
-      float x = 0.0f;
-#pragma unroll
-      for (int b = 0; b < R; ++b) x = fmaf(S0[b], rho[b], x);
-      float wt;
-      if (g.w) {
-        wt = g.w[t];
+        float wt = yt;
+        if (!g.w) {
+          const double res = (double)v[0] - (double)yt;
+          lsum += 0.5 * res * res;
+          wt = (float)res;
+        }
+        Wt[tt] = wt;
       } else {
-        const double res = (double)x - (double)g.y[t];
-        lsum += 0.5 * res * res;
-        wt = (float)res;
-      }
-      float l[R];
+        for (int k = 0; k < d; ++k) {
+          const int sl = IDX[k * T + tt];
+          const int p = WC[(k * NB + sl) * NW + tw] + RANK[k * T + tt];
+          TID[k * T + p] = (unsigned char)tt;
+          if (k > 0)
 #pragma unroll
-      for (int a = 0; a < R; ++a) l[a] = a == 0 ? wt : 0.0f;
-      for (int k = 0; k < d; ++k) {
-        const int p = POS[k * T + tid];
+            for (int h = 0; h < H; ++h)
+              LW[((size_t)(k - 1) * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+          if (k + 1 == d) break;
+          const float* S = Ls + (k * nmax + sl) * SS;
+          float nl[R];
 #pragma unroll
-        for (int h = 0; h < H; ++h)
-          LW[((size_t)k * H + h) * T + p] = make_float4(l[4 * h], l[4 * h + 1], l[4 * h + 2], l[4 * h + 3]);
-        if (k + 1 == d) break;
-        const float* S = Ls + (k * nmax + IDX[k * T + tid]) * SS;
-        float nl[R];
+          for (int b = 0; b < R; ++b) nl[b] = 0.0f;
 #pragma unroll
-        for (int b = 0; b < R; ++b) nl[b] = 0.0f;
+          for (int a = 0; a < R; ++a) {
 #pragma unroll
-        for (int a = 0; a < R; ++a) {
-#pragma unroll
-          for (int b = 0; b < R; b += 4) {
-            const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
-            nl[b] = fmaf(l[a], s4.x, nl[b]);
-            nl[b + 1] = fmaf(l[a], s4.y, nl[b + 1]);
-            nl[b + 2] = fmaf(l[a], s4.z, nl[b + 2]);
-            nl[b + 3] = fmaf(l[a], s4.w, nl[b + 3]);
+            for (int b = 0; b < R; b += 4) {
+              const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+              nl[b] = fmaf(v[a], s4.x, nl[b]);
+              nl[b + 1] = fmaf(v[a], s4.y, nl[b + 1]);
+              nl[b + 2] = fmaf(v[a], s4.z, nl[b + 2]);
+              nl[b + 3] = fmaf(v[a], s4.w, nl[b + 3]);
+            }
           }
-        }
 #pragma unroll
-        for (int b = 0; b < R; ++b) l[b] = nl[b];
+          for (int b = 0; b < R; ++b) v[b] = nl[b];
+        }
       }
     }
     __syncthreads();
-    // (3) accumulation: this thread's item over its share of the bucket
+    // (3) accumulation: this thread's item over its share of the bucket (l = 1 before the first
+    // core, rho = 1 after the last)
     if (ik >= 0) {
-      const int p0 = BO[ik * (NB + 1) + is], p1 = BO[ik * (NB + 1) + is + 1];
-      const float4* lw = LW + (size_t)ik * H * T;
+      const int p0 = BO[ik * NB + is], p1 = BO[ik * NB + is + 1];
+      const unsigned char* tb = TID + (size_t)ik * T;
+      const float4* lw = LW + (size_t)(ik - 1) * H * T;
       const float4* rh = RH + (size_t)ik * H * T;
-      if (ik == 0 || ik == d - 1) {
+      if (ik == 0) {
         for (int p = p0 + ip; p < p1; p += np) {
-          float lv[R], rv[R];
+          const float w = Wt[tb[p]];
+          if (d == 1) {
+            acc[0][0] += w;
+            continue;
+          }
+#pragma unroll
+          for (int h = 0; h < H; ++h) {
+            const float4 b4 = rh[(size_t)h * T + p];
+            acc[0][4 * h] = fmaf(w, b4.x, acc[0][4 * h]);
+            acc[0][4 * h + 1] = fmaf(w, b4.y, acc[0][4 * h + 1]);
+            acc[0][4 * h + 2] = fmaf(w, b4.z, acc[0][4 * h + 2]);
+            acc[0][4 * h + 3] = fmaf(w, b4.w, acc[0][4 * h + 3]);
+          }
+        }
+      } else if (ik == d - 1) {
+        for (int p = p0 + ip; p < p1; p += np) {
+          const float w = Wt[tb[p]];
 #pragma unroll
           for (int h = 0; h < H; ++h) {
             const float4 a4 = lw[(size_t)h * T + p];
-            const float4 b4 = rh[(size_t)h * T + p];
-            lv[4 * h] = a4.x; lv[4 * h + 1] = a4.y; lv[4 * h + 2] = a4.z; lv[4 * h + 3] = a4.w;
-            rv[4 * h] = b4.x; rv[4 * h + 1] = b4.y; rv[4 * h + 2] = b4.z; rv[4 * h + 3] = b4.w;
-          }
-          if (ik == 0) {
-#pragma unroll
-            for (int b = 0; b < R; ++b) acc[0][b] = fmaf(lv[0], rv[b], acc[0][b]);
-          } else {
-#pragma unroll
-            for (int a = 0; a < R; ++a) acc[a][0] = fmaf(lv[a], rv[0], acc[a][0]);
+            acc[4 * h][0] = fmaf(w, a4.x, acc[4 * h][0]);
+            acc[4 * h + 1][0] = fmaf(w, a4.y, acc[4 * h + 1][0]);
+            acc[4 * h + 2][0] = fmaf(w, a4.z, acc[4 * h + 2][0]);
+            acc[4 * h + 3][0] = fmaf(w, a4.w, acc[4 * h + 3][0]);
           }
         }
       } else {
         for (int p = p0 + ip; p < p1; p += np) {
+          const float w = Wt[tb[p]];
           float lv[R], rv[R];
 #pragma unroll
           for (int h = 0; h < H; ++h) {
             const float4 a4 = lw[(size_t)h * T + p];
             const float4 b4 = rh[(size_t)h * T + p];
-            lv[4 * h] = a4.x; lv[4 * h + 1] = a4.y; lv[4 * h + 2] = a4.z; lv[4 * h + 3] = a4.w;
+            lv[4 * h] = w * a4.x; lv[4 * h + 1] = w * a4.y; lv[4 * h + 2] = w * a4.z; lv[4 * h + 3] = w * a4.w;
             rv[4 * h] = b4.x; rv[4 * h + 1] = b4.y; rv[4 * h + 2] = b4.z; rv[4 * h + 3] = b4.w;
           }
 #pragma unroll
@@ -555,10 +604,11 @@ __global__ void __launch_bounds__(256, 1) k_completion(const __grid_constant__ C
         }
       }
     }
-    __syncthreads();
   }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
   // sum the parts of every (core, slice) in shared memory, then write the CTA's partial
-  float* cacc = reinterpret_cast<float*>(RH);  // d * nmax * R * R floats (fits in RH)
+  float* cacc = reinterpret_cast<float*>(RH);  // d * nmax * R * R floats (fits the region)
   for (int e = tid; e < d * nmax * R * R; e += blockDim.x) cacc[e] = 0.0f;
   __syncthreads();
   if (ik >= 0) {
@@ -585,17 +635,39 @@ __global__ void __launch_bounds__(256, 1) k_completion(const __grid_constant__ C
     __syncthreads();
     if (tid == 0) {
       double s2 = 0.0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s2 += red[i];
+      for (int i = 0; i < nwarps; ++i) s2 += red[i];
       g.loss_part[blockIdx.x] = s2;
     }
   }
 }
 
-__global__ void k_reduce_partials(const float* part, int nparts, long long size, float* out) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < size;
-       e += (long long)gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int p = 0; p < nparts; ++p) s += part[(long long)p * size + e];
+// Sum of the per-CTA partials in a fixed order: a block owns 32 elements, its eight rows of 32
+// threads each sum every eighth partial and are then summed in order (one thread per element
+// over all partials left 21 of 608 blocks with 300 dependent reads each: 32 us, now 5 us). One
+// more block sums the loss partials where there is a loss.
+__global__ void __launch_bounds__(256) k_reduce_partials(const float* part, int nparts, long long size, float* out,
+                                                         const double* lpart, double* loss) {
+  __shared__ float sm[8][33];
+  __shared__ double red[8];
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+  const long long blocks = (size + 31) / 32;
+  if (blockIdx.x == blocks) {
+    double s = 0.0;
+    for (int p = threadIdx.x; p < nparts; p += 256) s += lpart[p];
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) *loss = s;
+    return;
+  }
+  const long long e = (long long)blockIdx.x * 32 + lane;
+  float s = 0.0f;
+  if (e < size)
+#pragma unroll 4
+    for (int p = row; p < nparts; p += 8) s += part[(long long)p * size + e];
+  sm[row][lane] = s;
+  __syncthreads();
+  if (row == 0 && e < size) {
+#pragma unroll
+    for (int r = 1; r < 8; ++r) s += sm[r][lane];
     out[e] = s;
   }
 }
@@ -634,57 +706,69 @@ struct GatherLayout {
   size_t smem;
   size_t loss_off, grad_off, total;
   // bucketed adjoint
-  int bucketed, T, NB;
+  int bucketed, T, NB, region;
   int parts[T3F_MAX_D];
   int item0[T3F_MAX_D + 1];
 };
 
-static size_t completion_smem(int d, int nmax, int R, int T, bool same) {
-  const size_t SS = (size_t)R * R + 4;
-  const int NB = nmax + 1, NW = (T + 31) / 32;
-  size_t b = sizeof(float) * ((same ? 1 : 2) * (size_t)d * nmax * SS + 2 * (size_t)d * R * T);
-  b += 2 * (size_t)d * T;                           // POS
-  b += ((size_t)d * T + 15) & ~(size_t)15;          // IDX
-  b += sizeof(unsigned short) * (((size_t)d * NB * NW + 1) & ~(size_t)1);  // WC (counts <= T)
-  b += sizeof(int) * ((size_t)d * NB + (size_t)d * (NB + 1));
-  return b;
+// Floats of the RH / LW region: both chains' vectors, the landing zone of the packed objects and the
+// final sums of the parts all use it.
+static long long completion_region(const TTV& L, const TTV& Rv, int R, int T, bool same) {
+  const long long nl = L.off[L.d - 1] + L.osz[L.d - 1], nr = same ? 0 : Rv.off[Rv.d - 1] + Rv.osz[Rv.d - 1];
+  long long f = std::max(2LL * (L.d - 1) * R * T, (long long)L.d * L.nmax * R * R);
+  f = std::max(f, nl + nr + 16);  // each rounded out to 16 bytes on both sides
+  return (f + 3) & ~3LL;
 }
 
-// Choose the bucketed adjoint when its items fit one CTA and its buffers fit shared memory:
-// the largest chunk T whose buffers let two CTAs share an SM (one CTA's barrier waits overlap
-// the other's chains), else the largest that fits one CTA.
-static bool plan_completion(const TTV& L, bool same, int R, GatherLayout* lay) {
+static size_t completion_smem(const TTV& L, const TTV& Rv, int R, int T, bool same) {
+  const size_t SS = (size_t)R * R + 4, d = L.d;
+  const size_t NB = L.nmax + 1, NW = T / 32;
+  size_t b = sizeof(float) * ((same ? 1 : 2) * d * L.nmax * SS + (size_t)completion_region(L, Rv, R, T, same) + T);
+  b += sizeof(int) * d * T;                              // IN
+  b += sizeof(unsigned short) * (d * NB * NW + d * NB);  // WC, BO (counts <= T)
+  b += 3 * d * T;                                        // IDX, RANK, TID
+  return (b + 15) & ~(size_t)15;
+}
+
+// Choose the bucketed adjoint when its items fit one CTA and its buffers fit shared memory: the
+// largest chunk T <= 256 of one CTA per SM, or the largest of two CTAs per SM (one CTA's barrier
+// waits overlap the other's chains) where that keeps three quarters of its tuples in flight.
+static bool plan_completion(const TTV& L, const TTV& Rv, bool same, int R, GatherLayout* lay) {
   if (R > 8 || L.nmax > 254) return false;
   const int d = L.d;
-  for (int pass = 0; pass < 2; ++pass)
-  for (int T = 256; T >= 128; T -= 32) {
-    if (L.nmax * R > T) continue;
-    // two CTAs per SM: 228 KB per SM less 1 KB reserved and the static block per CTA
-    const size_t cap = pass == 0 ? (228 * 1024 - 2 * 1200) / 2 : 220 * 1024;
-    if (completion_smem(d, L.nmax, R, T, same) > cap) continue;
-    // boundary cores take one item per slice, interior cores share the rest evenly
-    int bnd = 0, inner = 0;
-    for (int k = 0; k < d; ++k) {
-      if (k == 0 || k == d - 1) bnd += L.n[k];
-      else inner += L.n[k];
-    }
-    const int P2 = inner ? (T - bnd) / inner : 1;
-    if (P2 < 1) continue;
-    int it = 0;
-    for (int k = 0; k < d; ++k) {
-      lay->item0[k] = it;
-      lay->parts[k] = (k == 0 || k == d - 1) ? 1 : P2;
-      it += L.n[k] * lay->parts[k];
-    }
-    lay->item0[d] = it;
-    if (it > T) continue;
-    lay->bucketed = pass == 0 ? 2 : 1;  // CTAs per SM
-    lay->T = T;
-    lay->NB = L.nmax + 1;
-    lay->smem = completion_smem(d, L.nmax, R, T, same);
-    return true;
+  // boundary cores take one item per slice, interior cores share the rest of the 2 T threads evenly
+  int bnd = 0, inner = 0;
+  for (int k = 0; k < d; ++k) {
+    if (k == 0 || k == d - 1) bnd += L.n[k];
+    else inner += L.n[k];
   }
-  return false;
+  auto best = [&](size_t cap) {
+    for (int T = 256; T >= 64; T -= 32) {
+      if (completion_smem(L, Rv, R, T, same) > cap || bnd + inner > 2 * T) continue;
+      return T;
+    }
+    return 0;
+  };
+  // two CTAs per SM: 228 KB per SM less 1 KB reserved and the static block per CTA; 128 registers a
+  // thread leave room for two CTAs of up to 256 threads
+  const int T1 = best(220 * 1024), T2 = std::min(128, best((228 * 1024 - 2 * 1400) / 2));
+  if (!T1) return false;
+  const bool two = T2 > 0 && bnd + inner <= 2 * T2 && 8 * T2 >= 3 * T1;
+  const int T = two ? T2 : T1;
+  const int P2 = inner ? (2 * T - bnd) / inner : 1;
+  int it = 0;
+  for (int k = 0; k < d; ++k) {
+    lay->item0[k] = it;
+    lay->parts[k] = (k == 0 || k == d - 1) ? 1 : P2;
+    it += L.n[k] * lay->parts[k];
+  }
+  lay->item0[d] = it;
+  lay->bucketed = two ? 2 : 1;  // CTAs per SM
+  lay->T = T;
+  lay->NB = L.nmax + 1;
+  lay->region = (int)completion_region(L, Rv, R, T, same);
+  lay->smem = completion_smem(L, Rv, R, T, same);
+  return true;
 }
 
 static GatherLayout gather_layout(const TTV& L, const TTV& Rv, long long N, bool bwd, bool same) {
@@ -697,7 +781,7 @@ static GatherLayout gather_layout(const TTV& L, const TTV& Rv, long long N, bool
     const long long nfl = L.off[L.d - 1] + L.osz[L.d - 1];
     lay.smem = sizeof(float) * (size_t)L.d * nmax * (R * R + 4) + (size_t)((nfl * 4 + 12 + 15) / 16) * 16;
     lay.grid = gather_grid(N, num_sms() * 8);
-  } else if (lay.R && plan_completion(L, same, R, &lay)) {
+  } else if (lay.R && plan_completion(L, Rv, same, R, &lay)) {
     long long g = (N + lay.T - 1) / lay.T;
     if (g > (long long)num_sms() * lay.bucketed) g = (long long)num_sms() * lay.bucketed;
     lay.grid = (int)(g < 1 ? 1 : g);
@@ -759,12 +843,13 @@ static t3f_status launch_completion(const GatherArgs& g, const GatherLayout& lay
   ca.g = g;
   ca.T = lay.T;
   ca.NB = lay.NB;
+  ca.region = lay.region;
   for (int k = 0; k < g.d; ++k) ca.parts[k] = lay.parts[k];
   for (int k = 0; k <= g.d; ++k) ca.item0[k] = lay.item0[k];
   auto kern = k_completion<R>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.smem) != cudaSuccess)
     return T3F_ERR_CUDA;
-  kern<<<lay.grid, lay.T, lay.smem, s>>>(ca);
+  kern<<<lay.grid, 2 * lay.T, lay.smem, s>>>(ca);
   return launch_status();
 }
 
@@ -888,12 +973,10 @@ extern "C" t3f_status t3f_gather_backward(const t3f_tt* X, const int32_t* idx, i
     // written) and the gauge projection writes the output from there
     target = gp;
   }
-  k_reduce_partials<<<num_sms() * 4, 256, 0, s>>>(gp, lay.grid, g.gsize, target);
+  const bool with_loss = loss && !w;
+  k_reduce_partials<<<(unsigned)((g.gsize + 31) / 32 + (with_loss ? 1 : 0)), 256, 0, s>>>(gp, lay.grid, g.gsize, target,
+                                                                                        lp, loss);
   T3F_CHECK(launch_status());
-  if (loss && !w) {
-    k_reduce_loss<<<1, 1024, 0, s>>>(lp, lay.grid, loss);
-    T3F_CHECK(launch_status());
-  }
   if (riemannian) T3F_CHECK(run_gauge_project(vl, gp, out, s));
   return T3F_OK;
 }
