@@ -334,18 +334,19 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_bwd(const __grid_cons
 //  (1) a deterministic counting sort of the chunk's tuples by slice, for every core (warp
 //      match + per-warp prefix sums; each thread of a tuple takes every other core), giving each
 //      tuple its bucket position at core k; the next chunk's indices are fetched meanwhile;
-//  (2) the two threads of a tuple run its two chains at once: the suffix chain storing rho_{k+1}
-//      (and the value, residual and weight), the prefix chain storing l_k and the tuple's number,
-//      both in the bucket order of core k;
+//  (2) both chains step core by core in bucket order, T threads each: the thread of row p at core k
+//      reads l_k (rho_{k+1}), multiplies it by its slice -- the same slice for the neighbouring
+//      rows of its bucket, so a warp reads three or four slices instead of 32 random ones -- and
+//      writes the result to its tuple's row in the order of core k + 1 (k - 1);
 //  (3) thread per item (core k, slice s, part): a persistent R x R register accumulator
 //      adds w l_k rho_{k+1}^T over the item's share of the bucket; consecutive lanes read
 //      consecutive bucket rows.
 // No atomics in the loop; the per-CTA partial is summed in a fixed order by a second kernel.
-// The slices are read at the tuples' random indices (16 16-byte loads per 64 multiply-adds of a
-// chain step), so the kernel is bound by shared-memory reads and their latency: two threads a
-// tuple, three block barriers a chunk (eight before) and no index load on the path. 10^6
-// tuples, d = 10, n = 10, r = 8: 529 us with one thread per tuple and the prefix after the suffix,
-// now @CM@ us; with two sets of slices (the Riemannian form) 591 -> @CR@ us.
+// Bound by shared-memory wavefronts (a chain step reads R^2 slice values per tuple for as many
+// multiply-adds). 10^6 tuples, d = 10, n = 10, r = 8: 529 us with one thread per tuple walking both
+// chains through its own slices, 422 us with the chains on two threads (shared-memory pipe 71 %
+// busy, 5.8 wavefronts a request), now 405 us (66 %); with two sets of slices (the Riemannian form)
+// 591 -> 462 -> 452 us.
 struct CompletionArgs {
   GatherArgs g;
   int T;                      // tuples per chunk (half of blockDim.x)
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
   constexpr int SS = R * R + 4;  // padded slice stride (breaks same-bank slices)
   constexpr int H = R / 4;       // float4 planes of a rank vector
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = T >> 5, nwarps = blockDim.x >> 5;
-  const int grp = tid >= T ? 1 : 0, tt = tid - grp * T, tw = tt >> 5;  // chain (0 suffix, 1 prefix), tuple, its warp
+  const int grp = tid >= T ? 1 : 0, tt = tid - grp * T, tw = tt >> 5;  // chain (0 suffix, 1 prefix), tuple / row, its warp
   const int SL = d * nmax * SS;
   float* Ls = sm;
   float* Rs = g.same ? Ls : Ls + SL;
@@ -374,9 +375,10 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
   int* IN = reinterpret_cast<int*>(Wt + T);                                // [d][T] the next chunk's indices
   unsigned short* WC = reinterpret_cast<unsigned short*>(IN + (size_t)d * T);  // [d][NB][NW]
   unsigned short* BO = WC + (size_t)d * NB * NW;                               // [d][NB] bucket starts
-  unsigned char* IDX = reinterpret_cast<unsigned char*>(BO + (size_t)d * NB);  // [d][T]
-  unsigned char* RANK = IDX + (size_t)d * T;                                   // [d][T]
-  unsigned char* TID = RANK + (size_t)d * T;                                   // [d][T] tuple of a bucket row
+  unsigned char* IDX = reinterpret_cast<unsigned char*>(BO + (size_t)d * NB);  // [d][T] slice of a tuple
+  unsigned char* POS = IDX + (size_t)d * T;   // [d][T] rank among its warp's, then bucket row of a tuple
+  unsigned char* TID = POS + (size_t)d * T;   // [d][T] tuple of a bucket row
+  unsigned char* SLC = TID + (size_t)d * T;   // [d][T] slice of a bucket row
 
   // stage the cores as zero-padded R x R slices with stride SS: the whole object(s) land in
   // the RH / LW region (not used before the first chunk) through one TMA bulk copy each
@@ -424,6 +426,7 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
   for (long long base = (long long)blockIdx.x * T; base < g.N; base += (long long)gridDim.x * T) {
     const long long t = base + tt;
     const bool valid = t < g.N;
+    const int nv = (int)min((long long)T, g.N - base);  // valid tuples: the first nv rows of every core
     float yt = 0.0f;
     if (grp == 0 && valid) yt = g.w ? __ldg(g.w + t) : __ldg(g.y + t);
     // (1) counting sort by slice (the counts of a (core, warp) belong to that warp)
@@ -441,12 +444,13 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
       const unsigned m = __match_any_sync(0xffffffffu, sl);
       const int rank = __popc(m & ((1u << lane) - 1u));
       IDX[k * T + tt] = (unsigned char)sl;
-      RANK[k * T + tt] = (unsigned char)rank;
+      POS[k * T + tt] = (unsigned char)rank;
       __syncwarp();
       if (rank == 0) WC[(k * NB + sl) * NW + tw] = (unsigned short)__popc(m);
     }
     fetch(base + (long long)gridDim.x * T);
     __syncthreads();  // counts complete; the previous chunk's accumulation is done
+    if (grp == 0) Wt[tt] = yt;
     for (int k = warp; k < d; k += nwarps) {  // a warp per core: scan over the slices
       int carry = 0;
       for (int b0 = 0; b0 < NB; b0 += 32) {
@@ -474,80 +478,103 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
       }
     }
     __syncthreads();
-    // (2) the tuple's chains; p = its row in the bucket order of core k
-    if (valid) {
-      float v[R];
+    for (int k = grp; k < d; k += 2) {
+      const int sl = IDX[k * T + tt], p = WC[(k * NB + sl) * NW + tw] + POS[k * T + tt];
+      POS[k * T + tt] = (unsigned char)p;
+      TID[k * T + p] = (unsigned char)tt;
+      SLC[k * T + p] = (unsigned char)sl;
+    }
+    __syncthreads();
+    // (2) the chains, row tt of each core in turn
+    for (int q = 0; q + 1 < d; ++q) {
+      if (tt < nv) {
+        if (grp == 0) {
+          const int k = d - 1 - q;
+          const float* S = Rs + (k * nmax + SLC[k * T + tt]) * SS;
+          const int p = POS[(k - 1) * T + TID[k * T + tt]];
+          float v[R], nr[R];
+          if (q == 0) {
 #pragma unroll
-      for (int a = 0; a < R; ++a) v[a] = a == 0 ? 1.0f : 0.0f;
-      if (grp == 0) {
-        for (int k = d - 1; k >= 0; --k) {
-          const int sl = IDX[k * T + tt];
-          const float* S = Rs + (k * nmax + sl) * SS;
-          if (k < d - 1) {
-            const int p = WC[(k * NB + sl) * NW + tw] + RANK[k * T + tt];
+            for (int a = 0; a < R; ++a) nr[a] = S[a * R];
+          } else {
 #pragma unroll
-            for (int h = 0; h < H; ++h)
-              RH[((size_t)k * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
-          }
-          if (k == 0) {
-            float x = 0.0f;
-#pragma unroll
-            for (int b = 0; b < R; ++b) x = fmaf(S[b], v[b], x);
-            v[0] = x;
-            break;
-          }
-          float nr[R];
-#pragma unroll
-          for (int a = 0; a < R; ++a) {
-            float acc1 = 0.0f;
-#pragma unroll
-            for (int b = 0; b < R; b += 4) {
-              const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
-              acc1 = fmaf(s4.x, v[b], acc1);
-              acc1 = fmaf(s4.y, v[b + 1], acc1);
-              acc1 = fmaf(s4.z, v[b + 2], acc1);
-              acc1 = fmaf(s4.w, v[b + 3], acc1);
+            for (int h = 0; h < H; ++h) {
+              const float4 r4 = RH[((size_t)k * H + h) * T + tt];
+              v[4 * h] = r4.x; v[4 * h + 1] = r4.y; v[4 * h + 2] = r4.z; v[4 * h + 3] = r4.w;
             }
-            nr[a] = acc1;
-          }
 #pragma unroll
-          for (int a = 0; a < R; ++a) v[a] = nr[a];
-        }
-        float wt = yt;
-        if (!g.w) {
-          const double res = (double)v[0] - (double)yt;
-          lsum += 0.5 * res * res;
-          wt = (float)res;
-        }
-        Wt[tt] = wt;
-      } else {
-        for (int k = 0; k < d; ++k) {
-          const int sl = IDX[k * T + tt];
-          const int p = WC[(k * NB + sl) * NW + tw] + RANK[k * T + tt];
-          TID[k * T + p] = (unsigned char)tt;
-          if (k > 0)
+            for (int a = 0; a < R; ++a) {
+              float acc1 = 0.0f;
 #pragma unroll
-            for (int h = 0; h < H; ++h)
-              LW[((size_t)(k - 1) * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
-          if (k + 1 == d) break;
-          const float* S = Ls + (k * nmax + sl) * SS;
-          float nl[R];
-#pragma unroll
-          for (int b = 0; b < R; ++b) nl[b] = 0.0f;
-#pragma unroll
-          for (int a = 0; a < R; ++a) {
-#pragma unroll
-            for (int b = 0; b < R; b += 4) {
-              const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
-              nl[b] = fmaf(v[a], s4.x, nl[b]);
-              nl[b + 1] = fmaf(v[a], s4.y, nl[b + 1]);
-              nl[b + 2] = fmaf(v[a], s4.z, nl[b + 2]);
-              nl[b + 3] = fmaf(v[a], s4.w, nl[b + 3]);
+              for (int b = 0; b < R; b += 4) {
+                const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+                acc1 = fmaf(s4.x, v[b], acc1);
+                acc1 = fmaf(s4.y, v[b + 1], acc1);
+                acc1 = fmaf(s4.z, v[b + 2], acc1);
+                acc1 = fmaf(s4.w, v[b + 3], acc1);
+              }
+              nr[a] = acc1;
             }
           }
 #pragma unroll
-          for (int b = 0; b < R; ++b) v[b] = nl[b];
+          for (int h = 0; h < H; ++h)
+            RH[((size_t)(k - 1) * H + h) * T + p] = make_float4(nr[4 * h], nr[4 * h + 1], nr[4 * h + 2], nr[4 * h + 3]);
+        } else {
+          const int k = q;
+          const float* S = Ls + (k * nmax + SLC[k * T + tt]) * SS;
+          const int p = POS[(k + 1) * T + TID[k * T + tt]];
+          float v[R], nl[R];
+          if (q == 0) {
+#pragma unroll
+            for (int b = 0; b < R; ++b) nl[b] = S[b];
+          } else {
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+              const float4 l4 = LW[((size_t)(k - 1) * H + h) * T + tt];
+              v[4 * h] = l4.x; v[4 * h + 1] = l4.y; v[4 * h + 2] = l4.z; v[4 * h + 3] = l4.w;
+            }
+#pragma unroll
+            for (int b = 0; b < R; ++b) nl[b] = 0.0f;
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+#pragma unroll
+              for (int b = 0; b < R; b += 4) {
+                const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+                nl[b] = fmaf(v[a], s4.x, nl[b]);
+                nl[b + 1] = fmaf(v[a], s4.y, nl[b + 1]);
+                nl[b + 2] = fmaf(v[a], s4.z, nl[b + 2]);
+                nl[b + 3] = fmaf(v[a], s4.w, nl[b + 3]);
+              }
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < H; ++h)
+            LW[((size_t)k * H + h) * T + p] = make_float4(nl[4 * h], nl[4 * h + 1], nl[4 * h + 2], nl[4 * h + 3]);
         }
+      }
+      __syncthreads();
+    }
+    // the value (from the suffix cores), residual and weight of row tt of the first core
+    if (grp == 0 && tt < nv) {
+      const float* S = Rs + SLC[tt] * SS;
+      const int o = TID[tt];
+      float x = S[0];
+      if (d > 1) {
+        x = 0.0f;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const float4 r4 = RH[(size_t)h * T + tt];
+          const float4 s4 = *reinterpret_cast<const float4*>(S + 4 * h);
+          x = fmaf(s4.x, r4.x, x);
+          x = fmaf(s4.y, r4.y, x);
+          x = fmaf(s4.z, r4.z, x);
+          x = fmaf(s4.w, r4.w, x);
+        }
+      }
+      if (!g.w) {
+        const double res = (double)x - (double)Wt[o];
+        lsum += 0.5 * res * res;
+        Wt[o] = (float)res;
       }
     }
     __syncthreads();
@@ -726,7 +753,7 @@ static size_t completion_smem(const TTV& L, const TTV& Rv, int R, int T, bool sa
   size_t b = sizeof(float) * ((same ? 1 : 2) * d * L.nmax * SS + (size_t)completion_region(L, Rv, R, T, same) + T);
   b += sizeof(int) * d * T;                              // IN
   b += sizeof(unsigned short) * (d * NB * NW + d * NB);  // WC, BO (counts <= T)
-  b += 3 * d * T;                                        // IDX, RANK, TID
+  b += 4 * d * T;                                        // IDX, POS, TID, SLC
   return (b + 15) & ~(size_t)15;
 }
 
