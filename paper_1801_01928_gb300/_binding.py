@@ -7,7 +7,10 @@ status. All arithmetic runs in the library's CUDA kernels; there is no fallback 
 """
 from __future__ import annotations
 
+import array
 import ctypes
+import functools
+import itertools
 import os
 from typing import Optional, Sequence
 
@@ -121,6 +124,13 @@ def _i32(vals: Sequence[int]):
     return (ctypes.c_int32 * len(vals))(*[int(v) for v in vals])
 
 
+@functools.lru_cache(maxsize=1024)
+def _i32_of(vals: tuple):
+    """The C array of a shape tuple. The library only reads it, so calls of equal shape share one
+    (a descriptor took 3.7 us to build, a third of a small call's host time went into them)."""
+    return (ctypes.c_int32 * len(vals))(*vals)
+
+
 class TT:
     """A batch of TT-vectors (m is None) or TT-matrices in the library's packed layout.
 
@@ -185,8 +195,8 @@ class TT:
         return _CODE[self.data.dtype]
 
     def desc(self) -> _Desc:
-        n, r = _i32(self.n), _i32(self.ranks)
-        m = _i32(self.m) if self.m is not None else None
+        n, r = _i32_of(tuple(self.n)), _i32_of(tuple(self.ranks))
+        m = _i32_of(tuple(self.m)) if self.m is not None else None
         self._keep = (n, r, m)
         return _Desc(self.batch, self.d, m if m is not None else None, n, r,
                      ctypes.c_void_p(self.data.data_ptr()), self.dtype_code)
@@ -196,9 +206,27 @@ def _ref(t: Optional[TT]):
     return None if t is None else ctypes.byref(t.desc())
 
 
+def _shape_key(t: Optional[TT]):
+    return None if t is None else (t.batch, tuple(t.n), tuple(t.ranks), None if t.m is None else tuple(t.m), t.dtype_code)
+
+
+@functools.lru_cache(maxsize=1024)
+def _ws_bytes(op: int, a, b, n_items: int, device_index: int) -> int:
+    """t3f_workspace_size by value: it depends on the shapes, the storage types, the item count
+    and the device's SM count, not on the buffers (their addresses are not null, nothing more)."""
+    def desc(k):
+        if k is None:
+            return None
+        batch, n, r, m, dt = k
+        return ctypes.byref(_Desc(batch, len(n), None if m is None else _i32_of(m), _i32_of(n), _i32_of(r),
+                                  ctypes.c_void_p(256), dt))
+    return int(_lib().t3f_workspace_size(op, desc(a), desc(b), n_items))
+
+
 def _ws(op: str, a: TT, b: Optional[TT], n_items: int, device) -> torch.Tensor:
-    nbytes = _lib().t3f_workspace_size(OP[op], ctypes.byref(a.desc()), _ref(b), int(n_items))
-    return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
+    index = torch.cuda.current_device() if device.type == "cuda" else -1
+    nbytes = _ws_bytes(OP[op], _shape_key(a), _shape_key(b), int(n_items), index)
+    return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
 
 
 def workspace(op: str, a: TT, b: Optional[TT] = None, n_items: int = 0) -> torch.Tensor:
@@ -213,8 +241,9 @@ def workspace(op: str, a: TT, b: Optional[TT] = None, n_items: int = 0) -> torch
 def gram(A: TT, B: TT, math: str = "fp32") -> torch.Tensor:
     dev = A.data.device
     G = torch.empty(A.batch, B.batch, dtype=torch.float32, device=dev)
-    ws = _ws("gram", A, B, 0, dev)
-    _check(_lib().t3f_gram(_ref(A), _ref(B), _ptr(G), MATH[math], _ptr(ws), ws.numel(), _stream(dev)), "t3f_gram")
+    ws = None if math == "fp32" else _ws("gram", A, B, 0, dev)  # (the error word of the tensor-core waits)
+    _check(_lib().t3f_gram(_ref(A), _ref(B), _ptr(G), MATH[math], _ptr(ws), 0 if ws is None else ws.numel(),
+                           _stream(dev)), "t3f_gram")
     return G
 
 
@@ -476,10 +505,13 @@ class RaggedTT:
         return out
 
     def desc(self) -> _RDesc:
-        d = _i32(self.dims)
-        n = _i32([v for m in self.modes for v in m])
-        r = _i32([v for rr in self.ranks for v in rr])
-        off = (ctypes.c_int64 * self.count)(*self.offsets)
+        def c(ctype, code, vals):  # one pass into a flat buffer, no per-element conversion in Python
+            a = array.array(code, vals)
+            return (ctype * len(a)).from_buffer(a)
+        d = c(ctypes.c_int32, "i", self.dims)
+        n = c(ctypes.c_int32, "i", itertools.chain.from_iterable(self.modes))
+        r = c(ctypes.c_int32, "i", itertools.chain.from_iterable(self.ranks))
+        off = c(ctypes.c_int64, "q", self.offsets)
         self._keep = (d, n, r, off)
         return _RDesc(self.count, d, n, r, off, ctypes.c_void_p(self.data.data_ptr()), _CODE[self.data.dtype])
 

@@ -8,8 +8,8 @@
                                  differentiated w.r.t. the Z cores and c with X held fixed
 
 Every forward and backward is one call into libt3f; the only arithmetic done here is the
-chain-rule scaling of a cotangent that is not exactly one (a scalar times a gradient
-array). The differentiable argument of each wrapper is the packed core buffer `TT.data`.
+chain-rule scaling by a cotangent (a scalar times a gradient array). The differentiable
+argument of each wrapper is the packed core buffer `TT.data`.
 """
 from __future__ import annotations
 
@@ -22,12 +22,10 @@ def _meta(t: B.TT):
     return (t.n, t.ranks, t.batch, t.m)
 
 
-def _scaled(g: torch.Tensor, s: torch.Tensor, like: torch.Tensor) -> torch.Tensor:
-    if s.numel() == 1 and float(s) == 1.0:
-        out = g
-    else:
-        out = g * s.to(g.dtype)
-    return out.to(like.dtype)
+def _scaled(g: torch.Tensor, s: torch.Tensor) -> torch.Tensor:
+    """g times the scalar cotangent s, in g's type (reading s on the host to skip a product by one
+    would wait for the whole forward pass)."""
+    return g * s
 
 
 class _CompletionLoss(torch.autograd.Function):
@@ -44,7 +42,7 @@ class _CompletionLoss(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gl):
         (g,) = ctx.saved_tensors
-        return _scaled(g, gl, g), None, None, None
+        return _scaled(g, gl), None, None, None
 
 
 class _Gram(torch.autograd.Function):

@@ -15,8 +15,11 @@
 // tensor-core math the sweeps over the tile list and the (tile, core, side) gradient items
 // run instead. Every call only enqueues memsets and kernels, so it can be captured in a CUDA
 // graph after one prepare.
-#include <algorithm>
 #include <math.h>
+
+#include <algorithm>
+#include <memory>
+#include <mutex>
 #include <vector>
 
 #include "t3f_internal.cuh"
@@ -518,6 +521,63 @@ t3f_status build_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, co
   return T3F_OK;
 }
 
+// Plans of recent calls. Every call needs the plan of its collection (workspace offsets, list
+// lengths, tile limits) and building one takes 1-2 ms of host time at 512 objects, as long as the
+// kernels of a small collection run. The plan is a function of the shapes, the tile table and the SM
+// count alone, so the last kPlanCache of them are kept, found by comparing those values in full
+// (13 thousand integers at 512 objects, some 10 us), shared by all threads and dropped oldest first.
+constexpr size_t kPlanCache = 8;
+
+t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, const int* tiles,
+                    std::shared_ptr<const Plan>* out) {
+  struct Entry {
+    std::vector<int32_t> key;
+    std::shared_ptr<const Plan> plan;
+    uint64_t used;
+  };
+  static std::mutex mu;
+  static std::vector<Entry> cache;
+  static uint64_t clock = 0;
+  bool readable = X && X->d && X->n && X->ranks && X->obj_off && X->cores && X->count >= 1 && ngroups >= 1 && gstart;
+  std::vector<int32_t> key;
+  if (readable) {
+    size_t sd = 0;
+    for (int o = 0; o < X->count && readable; ++o) {
+      readable = X->d[o] >= 1 && X->d[o] <= T3F_MAX_D;
+      sd += (size_t)X->d[o];
+    }
+    if (readable) {
+      const int head[4] = {X->count, ngroups, X->dtype, sm_count_gg()};
+      key.reserve(16 + 3 * (size_t)X->count + 2 * sd + X->count + ngroups);
+      key.insert(key.end(), head, head + 4);
+      for (int b = 0; b < kBuckets; ++b) key.push_back(tiles ? tiles[b] : kDefaultTiles[b]);
+      key.insert(key.end(), gstart, gstart + ngroups + 1);
+      key.insert(key.end(), X->d, X->d + X->count);
+      key.insert(key.end(), X->n, X->n + sd);
+      key.insert(key.end(), X->ranks, X->ranks + sd + X->count);
+      for (int o = 0; o < X->count; ++o) {
+        key.push_back((int32_t)(uint32_t)(uint64_t)X->obj_off[o]);
+        key.push_back((int32_t)(uint32_t)((uint64_t)X->obj_off[o] >> 32));
+      }
+      std::lock_guard<std::mutex> lock(mu);
+      for (Entry& e : cache)
+        if (e.key == key) {
+          e.used = ++clock;
+          *out = e.plan;
+          return T3F_OK;
+        }
+    }
+  }
+  std::shared_ptr<Plan> plan = std::make_shared<Plan>();
+  T3F_CHECK(build_plan(X, ngroups, gstart, tiles, plan.get()));  // (refuses what was not readable)
+  *out = plan;
+  std::lock_guard<std::mutex> lock(mu);
+  if (cache.size() >= kPlanCache)
+    cache.erase(std::min_element(cache.begin(), cache.end(), [](const Entry& a, const Entry& b) { return a.used < b.used; }));
+  cache.push_back(Entry{std::move(key), *out, ++clock});
+  return T3F_OK;
+}
+
 // ---------------------------------------------------------------------------------------
 // small kernels: FP64 norms, pack / unpack of padded batches, cotangent gather
 // ---------------------------------------------------------------------------------------
@@ -563,8 +623,9 @@ using namespace t3f;
 
 extern "C" size_t t3f_gram_groups_workspace_size(const t3f_tt_ragged* X, int32_t ngroups, const int32_t* gstart,
                                                  const int32_t* tiles) {
-  Plan P;
-  if (build_plan(X, ngroups, gstart, tiles, &P) != T3F_OK) return 0;
+  std::shared_ptr<const Plan> plan;
+  if (get_plan(X, ngroups, gstart, tiles, &plan) != T3F_OK) return 0;
+  const Plan& P = *plan;
   return P.total;
 }
 
@@ -578,8 +639,9 @@ size_t gg_tc_scratch(const Plan& P, int math) {
 extern "C" size_t t3f_gram_groups_backward_workspace_size(const t3f_tt_ragged* X, int32_t ngroups,
                                                           const int32_t* gstart, const int32_t* tiles,
                                                           int32_t math) {
-  Plan P;
-  if (build_plan(X, ngroups, gstart, tiles, &P) != T3F_OK) return 0;
+  std::shared_ptr<const Plan> plan;
+  if (get_plan(X, ngroups, gstart, tiles, &plan) != T3F_OK) return 0;
+  const Plan& P = *plan;
   if (math == T3F_MATH_FP32) return P.total;
   if (math != T3F_MATH_TF32 && math != T3F_MATH_BF16) return 0;
   return P.total + gg_tc_scratch(P, math);
@@ -587,8 +649,9 @@ extern "C" size_t t3f_gram_groups_backward_workspace_size(const t3f_tt_ragged* X
 
 extern "C" t3f_status t3f_gram_groups_prepare(const t3f_tt_ragged* X, int32_t ngroups, const int32_t* gstart,
                                               const int32_t* tiles, void* ws, size_t ws_bytes, t3f_stream_t stream) {
-  Plan P;
-  T3F_CHECK(build_plan(X, ngroups, gstart, tiles, &P));
+  std::shared_ptr<const Plan> plan;
+  T3F_CHECK(get_plan(X, ngroups, gstart, tiles, &plan));
+  const Plan& P = *plan;
   T3F_CHECK(check_ws(ws, ws_bytes, P.total));
   return gg_tables_upload(P, static_cast<char*>(ws), (cudaStream_t)stream);
 }
@@ -596,8 +659,9 @@ extern "C" t3f_status t3f_gram_groups_prepare(const t3f_tt_ragged* X, int32_t ng
 extern "C" t3f_status t3f_gram_groups(const t3f_tt_ragged* X, int32_t ngroups, const int32_t* gstart,
                                       const int32_t* tiles, int32_t math, float* out, double* norms, void* ws,
                                       size_t ws_bytes, t3f_stream_t stream) {
-  Plan P;
-  T3F_CHECK(build_plan(X, ngroups, gstart, tiles, &P));
+  std::shared_ptr<const Plan> plan;
+  T3F_CHECK(get_plan(X, ngroups, gstart, tiles, &plan));
+  const Plan& P = *plan;
   T3F_CHECK(check_ws(ws, ws_bytes, P.total));
   if (!out) return T3F_ERR_ARG;
   if (math != T3F_MATH_FP32 && math != T3F_MATH_TF32 && math != T3F_MATH_BF16) return T3F_ERR_ARG;
@@ -636,8 +700,9 @@ extern "C" t3f_status t3f_gram_groups(const t3f_tt_ragged* X, int32_t ngroups, c
 extern "C" t3f_status t3f_gram_groups_backward(const t3f_tt_ragged* X, int32_t ngroups, const int32_t* gstart,
                                                const int32_t* tiles, int32_t math, const float* dout, float* dcores,
                                                void* ws, size_t ws_bytes, t3f_stream_t stream) {
-  Plan P;
-  T3F_CHECK(build_plan(X, ngroups, gstart, tiles, &P));
+  std::shared_ptr<const Plan> plan;
+  T3F_CHECK(get_plan(X, ngroups, gstart, tiles, &plan));
+  const Plan& P = *plan;
   if (math != T3F_MATH_FP32 && math != T3F_MATH_TF32 && math != T3F_MATH_BF16) return T3F_ERR_ARG;
   if (math == T3F_MATH_TF32 && X->dtype != T3F_F32) return T3F_ERR_DTYPE;
   T3F_CHECK(check_ws(ws, ws_bytes, P.total + (math == T3F_MATH_FP32 ? 0 : gg_tc_scratch(P, math))));
