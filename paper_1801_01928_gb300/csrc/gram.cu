@@ -203,6 +203,7 @@ static size_t ws_gram_bwd_generic(const TTV& A, const TTV& B) {
 }
 
 size_t ws_gram_bwd(const TTV& A, const TTV& B) {
+  if (gram_low_bwd_supported(A, B)) return ws_gram_low_bwd(A, B);
   return gram_tile_bwd_supported(A, B) ? ws_gram_tile_bwd(A, B) : ws_gram_bwd_generic(A, B);
 }
 
@@ -266,6 +267,7 @@ extern "C" t3f_status t3f_gram(const t3f_tt* A, const t3f_tt* B, float* G, int32
     if (err && cudaMemsetAsync(err, 0, sizeof(int), (cudaStream_t)stream) != cudaSuccess) return T3F_ERR_CUDA;
     return run_gram_mma(va, vb, G, math, err, (cudaStream_t)stream);
   }
+  if (gram_low_supported(va, vb)) return run_gram_low(va, vb, G, (cudaStream_t)stream);
   if (gram_tile_supported(va, vb)) return run_gram_tile(va, vb, G, (cudaStream_t)stream);
   return run_pair_sweep(va, vb, 0, G, nullptr, nullptr, (cudaStream_t)stream);
 }
@@ -323,6 +325,7 @@ extern "C" t3f_status t3f_gram_backward(const t3f_tt* A, const t3f_tt* B, const 
   if (args.dB && cudaMemsetAsync(args.dB, 0, sizeof(float) * t3f_packed_size(dB), s) != cudaSuccess)
     return T3F_ERR_CUDA;
   if (!args.dA && !args.dB) return T3F_OK;
+  if (gram_low_bwd_supported(va, vb)) return run_gram_low_bwd(va, vb, dG, args.dA, args.dB, ws, ws_bytes, s);
   if (gram_tile_bwd_supported(va, vb)) return run_gram_tile_bwd(va, vb, dG, args.dA, args.dB, ws, ws_bytes, s);
   return gram_bwd_accumulate(va, vb, dG, args.dA, args.dB, ws, ws_bytes, s);
 }

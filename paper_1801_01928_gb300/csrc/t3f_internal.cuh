@@ -209,6 +209,14 @@ t3f_status run_gram_tile(const TTV& A, const TTV& B, float* out, cudaStream_t s)
 bool gram_mma_supported(const TTV& A, const TTV& B, int math);
 t3f_status run_gram_mma(const TTV& A, const TTV& B, float* out, int math, int* err, cudaStream_t s);
 
+// Gram sweep and adjoint of uniform batches with ranks <= 16, F32 (gram_low.cu).
+bool gram_low_supported(const TTV& A, const TTV& B);
+bool gram_low_bwd_supported(const TTV& A, const TTV& B);
+t3f_status run_gram_low(const TTV& A, const TTV& B, float* out, cudaStream_t s);
+size_t ws_gram_low_bwd(const TTV& A, const TTV& B);
+t3f_status run_gram_low_bwd(const TTV& A, const TTV& B, const float* dG, float* dA, float* dB, void* ws,
+                            size_t ws_bytes, cudaStream_t s);
+
 // Tiled Gram adjoint (gram_tile_bwd.cu).
 bool gram_tile_bwd_supported(const TTV& A, const TTV& B);
 size_t ws_gram_tile_bwd(const TTV& A, const TTV& B);
