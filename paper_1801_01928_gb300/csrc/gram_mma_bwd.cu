@@ -29,12 +29,20 @@ namespace t3f {
 namespace {
 
 // Roles: warps 0-3 stage the y side's slices, warp 4 (one lane) issues the products, warps 5-8
-// (one per tensor-memory lane quarter) run the epilogues (and, for BF16, copy T to shared
-// memory). Slices, T and the gradient product are double-buffered, so slice i+1's first
-// product runs while slice i's second product and epilogue are in flight.
-constexpr int kGThreads = 288;
+// (one per tensor-memory lane quarter) copy T to shared memory (BF16), warps 9-12 and 13-16 add
+// the gradient products of even and odd slices to memory. Slices, T and the gradient product are
+// double-buffered, so slice i+1's first product runs while slice i's second product, copy and
+// additions are in flight. Nothing is near a rate: an item of n slices takes 3 us of loads and tables
+// and 2 us a slice, most of it the issue of 16 small products by one lane and waits between roles.
+// 512 objects of ranks 2 .. 64 in groups of 64, BF16: 3291 us with the copy of T and the additions (32
+// sectors an instruction) on the same four warps, 3488 with the additions coalesced, 2465 on warps
+// of their own, 2397 with one commit a product; uniform 100 x 100 pairs, d = n = 10, with the sweeps:
+// rank 16 1020 -> 887, rank 32 5020 -> 3960, rank 64 34893 -> 24191 (TF32 1225 -> 1213, 6326 -> 5521,
+// 39619 -> 29983).
+constexpr int kGThreads = 544;
 constexpr int kGProd = 128;           // staging threads (warps 0-3)
 constexpr int kGMmaWarp = 4;
+constexpr int kGAddWarp = 9;
 constexpr uint32_t kGTmemCols = 512;  // T[b] at columns 128 b, the gradient product Q[b] at 256 + 128 b
 
 struct GradTcArgs {
@@ -65,10 +73,12 @@ struct GradTcArgs {
 
 struct GradShared {
   uint64_t ld;                    // the two partial copies of an item
-  uint64_t sfull[2], sempty[2];   // slice ring: staged / read by the first product
-  uint64_t tdone[2], tfree[2];    // T buffers: written / consumed
-  uint64_t tsfull[2], tsfree[2];  // BF16 shared-memory copies of T: written / read
-  uint64_t qdone[2], qfree[2];    // gradient product buffers: written / read by the epilogue
+  // (a commit costs the issuing lane some 200 cycles, so one barrier tells everything that the end of a
+  // product frees)
+  uint64_t sfull[2];              // slice ring: staged
+  uint64_t tdone[2];              // T buffers: written, and the slice buffers read
+  uint64_t tfree[2], tsfull[2];   // BF16: T buffers copied, their shared-memory copies written
+  uint64_t qdone[2], qfree[2];    // gradient product buffers: written (and T, or its copy, read) / added
   uint64_t fin;                   // drain after a timeout
   long long ybase[8], xbase[8];
   int yrl[8], yrr[8], xrl[8], xrr[8];
@@ -111,11 +121,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// Shared-memory plan for element size es and y rank RY: gM, R, two slice buffers and (BF16)
-// two shared-memory copies of T.
+constexpr uint32_t kGStg = 33;  // row pitch of an epilogue warp's 32 x 32 block
+
+// Shared-memory plan for element size es and y rank RY: gM, R, two slice buffers, (BF16) two
+// shared-memory copies of T, and a 32 x 32 block per epilogue warp.
 __host__ __device__ constexpr uint32_t grad_slot(int es) { return 128u * 128u * (uint32_t)es; }
 __host__ __device__ constexpr uint32_t grad_smem(int es, int RY) {
-  return 2u * grad_slot(es) + 2u * 128u * (uint32_t)RY * (uint32_t)es + (es == 2 ? 2u * grad_slot(es) : 0u);
+  return 2u * grad_slot(es) + 2u * 128u * (uint32_t)RY * (uint32_t)es + (es == 2 ? 2u * grad_slot(es) : 0u) +
+         8u * 32u * kGStg * 4u;
 }
 
 // One work item: the gradient of side `side` of a tile for core k. x0 / nx: the objects whose
@@ -205,7 +218,7 @@ __device__ bool grad_item(const GradTcArgs& g, char* sm, GradShared& sh, uint32_
     load_slice(0);
     for (int i = 0; i < n; ++i) {
       const uint32_t gg = gs + (uint32_t)i, b = gg & 1u;
-      if (gg >= 2u && !warp_wait(su32(&sh.sempty[b]), ((gg >> 1) - 1u) & 1u)) {
+      if (gg >= 2u && !warp_wait(su32(&sh.tdone[b]), ((gg >> 1) - 1u) & 1u)) {
         ok = false;
         break;
       }
@@ -228,7 +241,7 @@ __device__ bool grad_item(const GradTcArgs& g, char* sm, GradShared& sh, uint32_
         if (i < n) {
           const uint32_t gg = gs + (uint32_t)i, b = gg & 1u;
           ok = mbar_wait(su32(&sh.sfull[b]), (gg >> 1) & 1u);
-          if (ok && gg >= 2u) ok = mbar_wait(su32(&sh.tfree[b]), ((gg >> 1) - 1u) & 1u);
+          if (ok && gg >= 2u) ok = mbar_wait(su32(KIND == 0 ? &sh.qdone[b] : &sh.tfree[b]), ((gg >> 1) - 1u) & 1u);
           if (!ok) break;
           tc_after();
           // T[(x, xi), (y, et')] = sum_et gM[(x, xi), (y, et)] Y_y,i[et, et'] for every y
@@ -242,7 +255,6 @@ __device__ bool grad_item(const GradTcArgs& g, char* sm, GradShared& sh, uint32_
               mma<KIND>(tmem + b * 128u + (uint32_t)(y * RY), da, db, ID1, kk > 0 ? 1u : 0u);
             }
           mma_commit(su32(&sh.tdone[b]));
-          mma_commit(su32(&sh.sempty[b]));
         }
         if (i >= 1) {
           // T R^T over all x at once (N = 128, K = 128) into Q[bj]; only its diagonal blocks
@@ -264,80 +276,107 @@ __device__ bool grad_item(const GradTcArgs& g, char* sm, GradShared& sh, uint32_
             }
           }
           mma_commit(su32(&sh.qdone[bj]));
-          mma_commit(su32(KIND == 0 ? &sh.tfree[bj] : &sh.tsfree[bj]));
         }
       }
     }
     __syncwarp();
-  } else {
-    // ---- epilogue warps: lane quarter qd of tensor memory
-    const int qd = warp & 3, row = qd * 32 + lane, xr = row / RX, xi = row % RX;
-    constexpr int QCOLS = RX < 32 ? 32 : RX;  // columns of the x blocks this quarter's lanes cover
-    const int cstart = ((qd * 32) / RX) * RX;
-    const bool xok = xr < nx && xi < sh.xrl[xr];
-    const int xrr = sh.xrr[xr];
-    const long long xrow = sh.xbase[xr] + (long long)xi * n * xrr;
-    for (int i = 0; i <= n; ++i) {
-      if constexpr (KIND == 1) {
-        if (i < n) {
-          // T(i) -> shared memory (rows (x, xi), K = (y, et')), rounded to BF16
-          const uint32_t gg = gs + (uint32_t)i, b = gg & 1u;
-          if (!warp_wait(su32(&sh.tdone[b]), (gg >> 1) & 1u) ||
-              (gg >= 2u && !warp_wait(su32(&sh.tsfree[b]), ((gg >> 1) - 1u) & 1u))) {
-            ok = false;
-            break;
-          }
-          tc_after();
-          char* const dst = ts + b * SLOT;
+  } else if (warp < kGAddWarp) {
+    // ---- BF16: T(i) -> shared memory (rows (x, xi), K = (y, et')), rounded to BF16
+    if constexpr (KIND == 1) {
+      const int qd = warp & 3, row = qd * 32 + lane;
+      for (int i = 0; i < n; ++i) {
+        const uint32_t gg = gs + (uint32_t)i, b = gg & 1u;
+        if (!warp_wait(su32(&sh.tdone[b]), (gg >> 1) & 1u) ||
+            (gg >= 2u && !warp_wait(su32(&sh.qdone[b]), ((gg >> 1) - 1u) & 1u))) {
+          ok = false;
+          break;
+        }
+        tc_after();
+        char* const dst = ts + b * SLOT;
 #pragma unroll
-          for (int cc = 0; cc < 128; cc += 64) {
-            uint32_t r[2][32];
-            tmem_ld32_nw(tmem + b * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)cc, r[0]);
-            tmem_ld32_nw(tmem + b * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cc + 32), r[1]);
-            tmem_wait_ld();
+        for (int cc = 0; cc < 128; cc += 64) {
+          uint32_t r[2][32];
+          tmem_ld32_nw(tmem + b * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)cc, r[0]);
+          tmem_ld32_nw(tmem + b * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cc + 32), r[1]);
+          tmem_wait_ld();
 #pragma unroll
-            for (int hh = 0; hh < 8; ++hh) {
-              float u[8];
+          for (int hh = 0; hh < 8; ++hh) {
+            float u[8];
 #pragma unroll
-              for (int t = 0; t < 8; ++t) u[t] = __uint_as_float(r[hh >> 2][(hh & 3) * 8 + t]);
-              *reinterpret_cast<uint4*>(dst + (uint32_t)(row >> 3) * SBO + (uint32_t)((cc + hh * 8) / 8) * 128u +
-                                        (uint32_t)(row & 7) * 16u) = O::pack(u);
-            }
-          }
-          async_fence();
-          tc_before();
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(su32(&sh.tsfull[b]));
-            mbar_arrive(su32(&sh.tfree[b]));
+            for (int t = 0; t < 8; ++t) u[t] = __uint_as_float(r[hh >> 2][(hh & 3) * 8 + t]);
+            *reinterpret_cast<uint4*>(dst + (uint32_t)(row >> 3) * SBO + (uint32_t)((cc + hh * 8) / 8) * 128u +
+                                      (uint32_t)(row & 7) * 16u) = O::pack(u);
           }
         }
+        async_fence();
+        tc_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(su32(&sh.tsfull[b]));
+          mbar_arrive(su32(&sh.tfree[b]));
+        }
       }
-      const int j = KIND == 0 ? i : i - 1;  // slice whose epilogue runs now
-      if (j < 0 || j >= n) continue;
-      const uint32_t gj = gs + (uint32_t)j, bj = gj & 1u;
-      if (!warp_wait(su32(&sh.qdone[bj]), (gj >> 1) & 1u)) {
+    }
+  } else {
+    // ---- adding warps: lane quarter qd of the gradient product buffer `set`
+    const int qd = warp & 3;
+    const uint32_t set = (uint32_t)(warp - kGAddWarp) >> 2;
+    constexpr int QCOLS = RX < 32 ? 32 : RX;  // columns of the x blocks this quarter's lanes cover
+    const int cstart = ((qd * 32) / RX) * RX;
+    // the quarter's rows: NB objects (or half of one), rows xi0 .. of them
+    constexpr int NB = RX < 32 ? 2 : 1;
+    const int xi0 = (qd * 32) % RX;
+    float* const stg = reinterpret_cast<float*>(ts + (KIND == 1 ? 2 * SLOT : 0)) + (warp - kGAddWarp) * 32 * kGStg;
+    int xrl[NB], xrr[NB];  // rows and columns of an object here
+    float* xrow[NB];
+#pragma unroll
+    for (int o = 0; o < NB; ++o) {
+      const int x = (qd * 32) / RX + o;
+      xrl[o] = x < nx && outX ? min(sh.xrl[x] - xi0, 32) : 0;
+      xrr[o] = sh.xrr[x];
+      xrow[o] = outX + sh.xbase[x] + (long long)xi0 * n * xrr[o];
+    }
+    for (int j = (int)((gs ^ set) & 1u); j < n; j += 2) {
+      const uint32_t gj = gs + (uint32_t)j;
+      if (!warp_wait(su32(&sh.qdone[set]), (gj >> 1) & 1u)) {
         ok = false;
         break;
       }
       tc_after();
-      // lane (x, xi) adds its block's columns to dX_x[xi, j, :]
+      // the quarter's diagonal blocks, added to dX_x[xi, j, :] along the columns (through shared memory:
+      // lanes along the rows of tensor memory would send every lane's word to its own sector)
       uint32_t r[QCOLS / 32][32];
 #pragma unroll
       for (int h = 0; h < QCOLS / 32; ++h)
-        tmem_ld32_nw(tmem + 256u + bj * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cstart + h * 32), r[h]);
+        tmem_ld32_nw(tmem + 256u + set * 128u + ((uint32_t)(qd * 32) << 16) + (uint32_t)(cstart + h * 32), r[h]);
       tmem_wait_ld();
-      if (xok && outX) {
-        float* const dst = outX + xrow + (long long)j * xrr;
-#pragma unroll
-        for (int t = 0; t < QCOLS; ++t) {
-          const int c = cstart + t, xc = c / RX, xp = c % RX;
-          if (xc == xr && xp < xrr) atomicAdd(dst + xp, __uint_as_float(r[t >> 5][t & 31]));
-        }
-      }
       tc_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(su32(&sh.qfree[bj]));
+      if (lane == 0) mbar_arrive(su32(&sh.qfree[set]));
+#pragma unroll
+      for (int h = 0; h < QCOLS / 32; ++h) {
+#pragma unroll
+        for (int t = 0; t < 32; ++t) stg[lane * kGStg + t] = __uint_as_float(r[h][t]);
+        __syncwarp();
+#pragma unroll
+        for (int o = 0; o < NB; ++o) {
+          const int wd = min(32, xrr[o] - h * 32);  // columns of this half
+          if (wd > 0) {
+            const int lg = wd > 1 ? 32 - __clz(wd - 1) : 0;  // 2^lg lanes a row
+            const int col = lane & ((1 << lg) - 1), stp = 32 >> lg, r0 = lane >> lg;
+            float* dst = xrow[o] + (long long)(r0 * n + j) * xrr[o] + h * 32 + col;
+            const long long dstep = (long long)stp * n * xrr[o];
+            const float* src = stg + (o * 16 + r0) * kGStg + o * 16 + col;
+            const int cnt = col < wd && r0 < xrl[o] ? (xrl[o] - r0 + stp - 1) >> (5 - lg) : 0;
+#pragma unroll 8
+            for (int q = 0; q < cnt; ++q) {
+              atomicAdd(dst, src[q * stp * kGStg]);
+              dst += dstep;
+            }
+          }
+        }
+        __syncwarp();
+      }
     }
   }
   return ok;
@@ -356,11 +395,9 @@ __device__ __forceinline__ void grad_setup(GradShared& sh, char* sm, uint32_t by
     init(&sh.fin, 1);
     for (int b = 0; b < 2; ++b) {
       init(&sh.sfull[b], kGProd);
-      init(&sh.sempty[b], 1);
       init(&sh.tdone[b], 1);
-      init(&sh.tfree[b], KIND == 0 ? 1 : 4);
+      init(&sh.tfree[b], 4);
       init(&sh.tsfull[b], 4);
-      init(&sh.tsfree[b], 1);
       init(&sh.qdone[b], 1);
       init(&sh.qfree[b], 4);
     }
