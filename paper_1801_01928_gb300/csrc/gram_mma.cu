@@ -190,7 +190,7 @@ __device__ __forceinline__ void pipe_wait(MmaState& st, int which, int p) {
 }
 __device__ __forceinline__ void pipe_commit(MmaState& st, int which, int p) {
   const uint32_t bar = which == 1 ? (p ? st.b1[1] : st.b1[0]) : (p ? st.b2[1] : st.b2[0]);
-  if (threadIdx.x == 0) mma_commit(bar);
+  mma_commit(bar);
 }
 __device__ __forceinline__ void pipe_mark(MmaState& st, int which, int p) {
   bool& pd = which == 1 ? (p ? st.pd1[1] : st.pd1[0]) : (p ? st.pd2[1] : st.pd2[0]);
@@ -431,11 +431,13 @@ __device__ bool mma_tile_sync(const GramMmaArgs& g, char* sm, MmaState& st, int 
       async_fence();
       tc_before();
       if (__syncthreads_or(st.bad)) return false;
-      if (tid == 0) {
+      if (warp == 0) {
         tc_after();
-        issue_mma1(0, 0);
+        if (elect_one()) {
+          issue_mma1(0, 0);
+          pipe_commit(st, 1, 0);
+        }
       }
-      pipe_commit(st, 1, 0);
       pipe_mark(st, 1, 0);
       if (n > 1)
         load_slice(k, 1);
@@ -451,11 +453,13 @@ __device__ bool mma_tile_sync(const GramMmaArgs& g, char* sm, MmaState& st, int 
           tc_before();
           if (__syncthreads_or(st.bad)) return false;
           // slice i + 1's first product into the other T buffer (transposed in iteration i - 1)
-          if (tid == 0) {
+          if (warp == 0) {
             tc_after();
-            issue_mma1((i + 1) % 3, p ^ 1);
+            if (elect_one()) {
+              issue_mma1((i + 1) % 3, p ^ 1);
+              pipe_commit(st, 1, p ^ 1);
+            }
           }
-          pipe_commit(st, 1, p ^ 1);
           pipe_mark(st, 1, p ^ 1);
           if (i + 2 < n)
             load_slice(k, i + 2);
@@ -468,11 +472,13 @@ __device__ bool mma_tile_sync(const GramMmaArgs& g, char* sm, MmaState& st, int 
         async_fence();
         tc_before();
         if (__syncthreads_or(st.bad)) return false;
-        if (tid == 0) {
+        if (warp == 0) {
           tc_after();
-          issue_mma2(i % 3, p, i > 0);
+          if (elect_one()) {
+            issue_mma2(i % 3, p, i > 0);
+            pipe_commit(st, 2, p);
+          }
         }
-        pipe_commit(st, 2, p);
         pipe_mark(st, 2, p);
       }
       pipe_wait(st, 2, 0);
@@ -491,16 +497,18 @@ __device__ bool mma_tile_sync(const GramMmaArgs& g, char* sm, MmaState& st, int 
       tc_before();
       if (__syncthreads_or(st.bad)) return false;
       // ---- MMA1: T for every b (TMEM columns b*RB .. b*RB + RB - 1)
-      if (tid == 0) {
+      if (warp == 0) {
         tc_after();
         const uint64_t da = sdesc(su32(mop), SBOB), db = sdesc(su32(bsl + s * TB * SLB), SBOB);
+        if (elect_one()) {
 #pragma unroll
-        for (int b = 0; b < TB; ++b)
+          for (int b = 0; b < TB; ++b)
 #pragma unroll
-          for (int kk = 0; kk < RB / O::KI; ++kk)
-            mma<KIND>(st.tmem + (uint32_t)(b * RB), da + ((b * BIGB + kk * 2 * kLBO) >> 4),
-                      db + ((b * SLB + kk * 2 * kLBO) >> 4), ID1, kk > 0);
-        mma_commit(st.bar1);
+            for (int kk = 0; kk < RB / O::KI; ++kk)
+              mma<KIND>(st.tmem + (uint32_t)(b * RB), da + ((b * BIGB + kk * 2 * kLBO) >> 4),
+                        db + ((b * SLB + kk * 2 * kLBO) >> 4), ID1, kk > 0);
+          mma_commit(st.bar1);
+        }
       }
       st.pending1 = true;
       // ---- prefetch the next slice while the products run
@@ -524,16 +532,18 @@ __device__ bool mma_tile_sync(const GramMmaArgs& g, char* sm, MmaState& st, int 
       tc_before();
       if (__syncthreads_or(st.bad)) return false;
       // ---- MMA2: D_a += T_a A_a,i for every a (TMEM columns 128 + a*RA ..)
-      if (tid == 0) {
+      if (warp == 0) {
         tc_after();
         const uint64_t da = sdesc(su32(top), SBOA), db = sdesc(su32(asl + s * TA * SLA), SBOA);
+        if (elect_one()) {
 #pragma unroll
-        for (int a = 0; a < TA; ++a)
+          for (int a = 0; a < TA; ++a)
 #pragma unroll
-          for (int kk = 0; kk < RA / O::KI; ++kk)
-            mma<KIND>(st.tmem + 128u + (uint32_t)(a * RA), da + ((a * BIGA + kk * 2 * kLBO) >> 4),
-                      db + ((a * SLA + kk * 2 * kLBO) >> 4), ID2, (i > 0 || kk > 0) ? 1u : 0u);
-        mma_commit(st.bar2);
+            for (int kk = 0; kk < RA / O::KI; ++kk)
+              mma<KIND>(st.tmem + 128u + (uint32_t)(a * RA), da + ((a * BIGA + kk * 2 * kLBO) >> 4),
+                        db + ((a * SLA + kk * 2 * kLBO) >> 4), ID2, (i > 0 || kk > 0) ? 1u : 0u);
+          mma_commit(st.bar2);
+        }
       }
       st.pending2 = true;
     }
