@@ -241,7 +241,7 @@ t3f_status t3f_orth_ranks(int32_t d, const int32_t* n, const int32_t* ranks,
 
 /*
  * Orthogonal forms of X for the tangent space of the fixed-rank manifold (paper
- * Section 3.2): three Householder sweeps in FP64 (right-to-left on X, left-to-right on the
+ * Section 3.2): three QR sweeps in FP64 (right-to-left on X, left-to-right on the
  * result giving U, right-to-left on U giving V), every QR normalised to diag(R) >= 0.
  * U_1..U_{d-1} are left-orthogonal ((r_{k-1} n_k) x r_k unfoldings with orthonormal
  * columns), U_d carries X; V_2..V_d are right-orthogonal, V_1 carries X; full(U) = full(V)

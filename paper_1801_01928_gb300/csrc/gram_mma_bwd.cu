@@ -33,7 +33,7 @@ namespace {
 // the next items' tables. Slices, T and the gradient product are double-buffered and the items form a
 // ring, so every role runs ahead of the next as far as its buffers allow, across items too.
 // What bounds it: latency, an item's loads (64 KB) and a slice's chain of product, copy, product,
-// addition; the tensor cores work an eighth of the time. 512 objects of ranks 2 .. 64 in groups of 64,
+// addition; the tensor cores work a quarter of the time. 512 objects of ranks 2 .. 64 in groups of 64,
 // BF16: 3291 us with the copy of T and the additions (32 sectors an instruction) on the same four
 // warps and a barrier per item; 2397 with the additions coalesced, on warps of their own, and one
 // commit a product; 1997 with every lane of a waiting warp polling (one lane and a shuffle: 350 cycles
