@@ -15,7 +15,7 @@
 //   row role     R' += X B_i^T,  Y = R B_i^T,  dA_a,i = sum_b (g M) Y^T
 // a lane sums dB (dA) over its objects, the S sub-objects meet by shuffles and one atomic per
 // element and tile goes to the gradient. The left partials of every interface go through a scratch
-// area per tile (t R x t RP floats each, never more than the 4 x 4 block kernels' areas).
+// area per tile (t R x t RP floats each, a full batch's no more than the 4 x 4 block kernels').
 //
 // 100 x 100 pairs, d = 10, n = 10, r = 10: forward 388 us with 4 x 4 blocks on padded ranks (three
 // barriers per slice) -> 203 us, adjoint 1826 -> 783 us. Bound by the issue of the two or three warps a
