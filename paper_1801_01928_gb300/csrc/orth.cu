@@ -646,7 +646,9 @@ __device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int 
     const int R1p = a.R1[k - 1];
     const int rows = pv.r0 * pv.n;
     const int rq = (rows + P - 1) / P, q0 = rank * rq, nq = max(0, min(rows, q0 + rq) - q0);
-    const int ldw = c | 1;  // (rows are read across the lanes)
+    // rows are read across the lanes: an odd stride where it fits the W region (sized for stride
+    // T3F_MAX_RANK; c = 64 with 253 rows or more does not fit and keeps the even one)
+    const int ldw = nq * (c | 1) <= a.rows_per * T3F_MAX_RANK ? c | 1 : c;
     for (int e = tid; e < nq * c; e += nth) {
       const int q = e / c, b = e % c;
       s.W[q * ldw + b] = pb[(long long)(q0 + q) * R1p + b];
