@@ -63,8 +63,13 @@ const int kBucketMax[kBuckets] = {8, 16, 32, 64};
 // 6 x 50 2390 -> 2140; below the line 4 x 40 1808 -> 1825, 8 x 16 1204 -> 1210, 1 x 64 712 -> 709.
 constexpr int kManyObjects = 256;
 const int kDefaultTiles[kBuckets] = {10, 6, 3, 1}, kDefaultTilesMany[kBuckets] = {16, 16, 4, 2};
-inline int default_tile(int count, int bucket) {
-  return count >= kManyObjects ? kDefaultTilesMany[bucket] : kDefaultTiles[bucket];
+// The caps of a call. The small table passed by value is the exported default (the binding's
+// DEFAULT_TILES) and means the same plan as no table at all: a workspace prepared with the one is used
+// with the other.
+inline void tile_caps(int count, const int* tiles, int* tl) {
+  const bool given = tiles && !std::equal(kDefaultTiles, kDefaultTiles + kBuckets, tiles);
+  const int* from = given ? tiles : (count >= kManyObjects ? kDefaultTilesMany : kDefaultTiles);
+  std::copy(from, from + kBuckets, tl);
 }
 
 int sm_count_gg() { return device_sm_count(); }
@@ -121,10 +126,9 @@ t3f_status build_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, co
   if (X->dtype != T3F_F32 && X->dtype != T3F_BF16) return T3F_ERR_DTYPE;
   if (gstart[0] != 0 || gstart[ngroups] != X->count) return T3F_ERR_SHAPE;
   int tl[kBuckets];
-  for (int b = 0; b < kBuckets; ++b) {
-    tl[b] = tiles ? tiles[b] : default_tile(X->count, b);
+  tile_caps(X->count, tiles, tl);
+  for (int b = 0; b < kBuckets; ++b)
     if (tl[b] < 1 || tl[b] > 16) return T3F_ERR_ARG;
-  }
   const int cnt = X->count;
   P->count = cnt;
   P->ngroups = ngroups;
@@ -558,7 +562,9 @@ t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, cons
       const int head[4] = {X->count, ngroups, X->dtype, sm_count_gg()};
       key.reserve(16 + 3 * (size_t)X->count + 2 * sd + X->count + ngroups);
       key.insert(key.end(), head, head + 4);
-      for (int b = 0; b < kBuckets; ++b) key.push_back(tiles ? tiles[b] : default_tile(X->count, b));
+      int tl[kBuckets];
+      tile_caps(X->count, tiles, tl);
+      key.insert(key.end(), tl, tl + kBuckets);
       key.insert(key.end(), gstart, gstart + ngroups + 1);
       key.insert(key.end(), X->d, X->d + X->count);
       key.insert(key.end(), X->n, X->n + sd);
