@@ -151,15 +151,29 @@ struct LowSlices {
   }
 };
 
-// Row al of a product runs where the core has it; on a core whose ranks come up to R when padded to
-// four the test is left out (the operands are zero there), which lets the rows' loads run ahead.
-template <int R>
-__device__ __forceinline__ bool fills(int e) {
-  return ((e + 3) & ~3) >= R;
+// How a core's ranks lie to R. kExact: all R (those that a product sums over). kPadded: they come up to R
+// when padded to four, and its rows are run without a test (the operands are zero there), which lets
+// their loads run ahead. kCut: row al runs where the core has it. Zero on both sides: a partial is cut
+// to its core's ranks (keep) wherever it passes on to the next role or core, since an infinity in a
+// padded row or column meets a zero of the slice there and would reach the real ones as NaN (a pair
+// that overflows FP32 before its last core is +-inf). Bits are masked instead of selected: the products
+// were branched around behind a select (adjoint of 100 x 100 pairs of rank 9 1201 us, with masks 797,
+// without either 784; forward 201 against 199, rank 7 95 against 82).
+enum { kCut, kPadded, kExact };
+
+template <int R, class F>
+__device__ __forceinline__ void by_ranks(int lo, F f) {
+  if (lo == R) f(std::integral_constant<int, kExact>());
+  else if (((lo + 3) & ~3) >= R) f(std::integral_constant<int, kPadded>());
+  else f(std::integral_constant<int, kCut>());
 }
-template <bool FULL>
+template <int MODE>
 __device__ __forceinline__ bool row_on(int al, int e) {
-  return FULL || al < e;
+  return MODE != kCut || al < e;
+}
+template <int MODE = kPadded>
+__device__ __forceinline__ float keep(float v, bool real) {
+  return MODE == kPadded ? __uint_as_float(__float_as_uint(v) & (real ? 0xffffffffu : 0u)) : v;
 }
 
 // Left sweep over cores 0 .. kend - 1. On return acc holds the column role's last partial (of interface
@@ -191,19 +205,19 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
   __syncthreads();
   int c = 0;  // running slice
   for (int k = 0; k < kend; ++k) {
-    const int n = g.A.n[k], eA0 = g.A.r[k], eB0 = g.B.r[k];
+    const int n = g.A.n[k], eA0 = g.A.r[k], eA1 = g.A.r[k + 1], eB0 = g.B.r[k], eB1 = g.B.r[k + 1];
 #pragma unroll
     for (int o = 0; o < Low<R>::O; ++o)
 #pragma unroll
       for (int q = 0; q < R; ++q) acc[o][q] = 0.0f;
-    auto slices = [&](auto full) {
-      constexpr bool FULL = decltype(full)::value;
+    auto slices = [&](auto mode) {
+      constexpr int MODE = decltype(mode)::value;
       for (int i = 0; i < n; ++i, ++c) {
         const float* As = sl.ring + (c % L::RING) * 2 * L::W * L::OS;
         const float* Bs = As + L::W * L::OS;
         float* T = Ts + (c & 1) * L::MAT;
         // row role: a = w, alpha = x
-        if (on && w < na && row_on<FULL>(x, eA0))
+        if (on && w < na && row_on<MODE>(x, eA0))
 #pragma unroll
           for (int o = 0; o < Low<R>::O; ++o) {
             const int b = sub + o * S;
@@ -214,11 +228,13 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
             for (int q = 0; q < R; ++q) t[q] = 0.0f;
 #pragma unroll
             for (int be = 0; be < R; ++be)
-              if (row_on<FULL>(be, eB0)) {
+              if (row_on<MODE>(be, eB0)) {
                 ld_row<R>(br, Bb + be * RP);
 #pragma unroll
                 for (int q = 0; q < R; ++q) t[q] = fmaf(m[o][be], br[q], t[q]);
               }
+#pragma unroll
+            for (int q = 0; q < R; ++q) t[q] = keep<MODE>(t[q], x < eA0);
             st_row<R>(T + (w * R + x) * P + b * RP, t);
           }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -234,7 +250,7 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
             const float* tc = T + a * R * P + w * RP + x;
 #pragma unroll
             for (int al = 0; al < R; ++al)
-              if (row_on<FULL>(al, eA0)) {
+              if (row_on<MODE>(al, eA0)) {
                 float ar[R];
                 const float tv = tc[al * P];
                 ld_row<R>(ar, Aa + al * RP);
@@ -244,8 +260,7 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
           }
       }
     };
-    if (fills<R>(min(eA0, eB0))) slices(std::true_type());
-    else slices(std::false_type());
+    by_ranks<R>(min(eA0, eB0), slices);
     if (k + 1 == kend && !SAVE) break;
     // the columns of M' become the rows of the next core's M
     if (on && w < nb)
@@ -263,6 +278,8 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
         const int b = sub + o * S;
         if (b >= nb) continue;
         ld_row<R>(m[o], Ms + (w * R + x) * P + b * RP);
+#pragma unroll
+        for (int q = 0; q < R; ++q) m[o][q] = keep(m[o][q], x < eA1 && q < eB1);
         if (SAVE) st_row<R>(scr + ((size_t)(k + 1) * g.t * R + w * R + x) * (g.t * RP) + b * RP, m[o]);
       }
   }
@@ -342,8 +359,8 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
     for (int e = tid; e < na * R * nb * RP; e += blockDim.x) {
       const int col = e % (nb * RP), row = e / (nb * RP), q = col % RP;
       float v = 0.0f;
-      if (q < R) v = k == 0 ? (row % R == 0 && q == 0 ? 1.0f : 0.0f) : scr[((size_t)k * g.t * R + row) * (g.t * RP) + col];
-      Ms[row * P + col] = gs[(row / R) * nb + col / RP] * v;
+      if (q < R) v = k == 0 ? 1.0f : scr[((size_t)k * g.t * R + row) * (g.t * RP) + col];
+      Ms[row * P + col] = keep(gs[(row / R) * nb + col / RP] * v, q < eB0 && row % R < eA0);
     }
 #pragma unroll
     for (int o = 0; o < Low<R>::O; ++o)
@@ -351,8 +368,8 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
       for (int q = 0; q < R; ++q) racc[o][q] = 0.0f;
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();  // M complete, slice c has landed
-    auto slices = [&](auto full) {
-      constexpr bool FULL = decltype(full)::value;
+    auto slices = [&](auto mode) {
+      constexpr int MODE = decltype(mode)::value;
       for (int i = 0; i < n; ++i, ++c) {
         const float* As = sl.ring + (c % L::RING) * 2 * L::W * L::OS;
         const float* Bs = As + L::W * L::OS;
@@ -361,7 +378,7 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
         float grad[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) grad[q] = 0.0f;
-        if (on && w < nb && row_on<FULL>(x, eB1))
+        if (on && w < nb && row_on<MODE>(x, eB1))
 #pragma unroll
           for (int o = 0; o < Low<R>::O; ++o) {
             const int a = sub + o * S;
@@ -371,11 +388,11 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
             const float* mr = Ms + a * R * P + w * RP;
 #pragma unroll
             for (int al = 0; al < R; ++al)
-              if (row_on<FULL>(al, eA0)) {
+              if (row_on<MODE>(al, eA0)) {
                 float ar[R], mv[R];
                 ld_row<R>(ar, Aa + al * RP);
                 ld_row<R>(mv, mr + al * P);
-                const float xv = dot_row<R>(ar, rcol[o]);
+                const float xv = keep<MODE>(dot_row<R>(ar, rcol[o]), al < eA0 && x < eB1);
                 xc[al * P] = xv;
 #pragma unroll
                 for (int q = 0; q < R; ++q) grad[q] = fmaf(mv[q], xv, grad[q]);
@@ -405,24 +422,24 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
             const float* Bb = Bs + b * L::OS;
             float xr[R], y[R];
             ld_row<R>(xr, X + (w * R + x) * P + b * RP);
-            if (!FULL) {  // rows and columns past the ranks were not written
+            if (MODE == kCut) {  // rows and columns past the ranks were not written
 #pragma unroll
               for (int q = 0; q < R; ++q) xr[q] = x < eA0 && q < eB1 ? xr[q] : 0.0f;
             }
 #pragma unroll
             for (int be = 0; be < R; ++be) {
               y[be] = 0.0f;
-              if (row_on<FULL>(be, eB0)) {
+              if (row_on<MODE>(be, eB0)) {
                 float br[R];
                 ld_row<R>(br, Bb + be * RP);
                 racc[o][be] += dot_row<R>(br, xr);
-                y[be] = dot_row<R>(br, rrow[o]);
+                y[be] = keep<MODE>(dot_row<R>(br, rrow[o]), be < eB0);
               }
             }
             const float* mr = Ms + w * R * P + b * RP;
 #pragma unroll
             for (int al = 0; al < R; ++al)
-              if (row_on<FULL>(al, eA0)) {
+              if (row_on<MODE>(al, eA0)) {
                 float mv[R];
                 ld_row<R>(mv, mr + al * P);
                 grad[al] += dot_row<R>(mv, y);
@@ -440,8 +457,7 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
         }
       }
     };
-    if (fills<R>(min(min(eA0, eA1), min(eB0, eB1)))) slices(std::true_type());
-    else slices(std::false_type());
+    by_ranks<R>(min(min(eA0, eA1), min(eB0, eB1)), slices);
     if (k == 0) break;
     // R' : rows to columns through the X buffer that the last slice did not use
     float* Rs = Xs + (c & 1) * L::MAT;
@@ -449,9 +465,9 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
 #pragma unroll
       for (int o = 0; o < Low<R>::O; ++o) {
         const int b = sub + o * S;
-        if (b < nb) st_row<R>(Rs + (w * R + x) * P + b * RP, racc[o]);
 #pragma unroll
-        for (int q = 0; q < R; ++q) rrow[o][q] = racc[o][q];
+        for (int q = 0; q < R; ++q) rrow[o][q] = keep(racc[o][q], x < eA0 && q < eB0);
+        if (b < nb) st_row<R>(Rs + (w * R + x) * P + b * RP, rrow[o]);
       }
     __syncthreads();  // (also: every read of M is done)
     if (on && w < nb)
