@@ -291,7 +291,8 @@ t3f_status t3f_project_sum_backward(const t3f_tt* U, const t3f_tt* V, const t3f_
  *   dU_j,k = (I - U_k U_k^T) Zhat_j,k for k < d, dU_j,d = Zhat_j,d.
  * U, V: F32 orthogonal forms (batch 1, ranks <= T3F_MAX_RANK); Z: F32 batch with U's modes;
  * dU: F32 descriptor of batch Z->batch with U's ranks. Summing dU_j over j gives
- * t3f_project_sum's result.
+ * t3f_project_sum's result. A wait of the sweeps that runs out writes T3F_ERR_TIMEOUT into the
+ * workspace's error word.
  */
 t3f_status t3f_project(const t3f_tt* U, const t3f_tt* V, const t3f_tt* Z, const float* c,
                        t3f_tt* dU, void* ws, size_t ws_bytes, t3f_stream_t stream);

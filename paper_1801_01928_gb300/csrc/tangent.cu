@@ -1107,13 +1107,15 @@ extern "C" t3f_status t3f_project(const t3f_tt* U, const t3f_tt* V, const t3f_tt
   char* w = static_cast<char*>(ws);
   float* Lst = reinterpret_cast<float*>(w + l.offL);
   float* Rst = reinterpret_cast<float*>(w + l.offR);
+  int* err = static_cast<int*>(ws);
+  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return T3F_ERR_CUDA;
   if (psweep_supported(vu, vz)) {
     // both sweeps bring their slices in by bulk copies of slice-major copies of U and V
     float* XC = reinterpret_cast<float*>(w + l.offXT);
     const float* srcs[2] = {static_cast<const float*>(vu.p), static_cast<const float*>(vv.p)};
     T3F_CHECK(run_xslices(vu, srcs, 2u, 2, XC, s));
-    T3F_CHECK(run_psweep(vu, vz, 0, XC, nullptr, nullptr, Lst, nullptr, l.ioff, s));
-    T3F_CHECK(run_psweep(vv, vz, 1, XC + xslices_size(vu), nullptr, nullptr, Rst, nullptr, l.ioff, s));
+    T3F_CHECK(run_psweep(vu, vz, 0, XC, nullptr, nullptr, Lst, nullptr, l.ioff, s, err));
+    T3F_CHECK(run_psweep(vv, vz, 1, XC + xslices_size(vu), nullptr, nullptr, Rst, nullptr, l.ioff, s, err));
   } else {
     T3F_CHECK(run_pair_sweep(vu, vz, 0, nullptr, Lst, l.ioff, s));
     T3F_CHECK(run_pair_sweep(vv, vz, 1, nullptr, Rst, l.ioff, s));
