@@ -537,8 +537,20 @@ t3f_status build_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, co
 // lengths, tile limits) and building one takes 1-2 ms of host time at 512 objects, as long as the
 // kernels of a small collection run. The plan is a function of the shapes, the tile table and the SM
 // count alone, so the last kPlanCache of them are kept, found by comparing those values in full
-// (13 thousand integers at 512 objects, some 10 us), shared by all threads and dropped oldest first.
-constexpr size_t kPlanCache = 8;
+// (13 thousand integers at 512 objects, some 10 us), shared by all threads and dropped oldest first;
+// together they hold at most kPlanBytes (some 230 bytes an object of six cores: a collection of more
+// than 10^5 objects is planned on each call, which then is a small part of it).
+constexpr size_t kPlanCache = 8, kPlanBytes = 32u << 20;
+
+template <class T>
+size_t held(const std::vector<T>& v) {
+  return v.capacity() * sizeof(T);
+}
+size_t held(const Plan& P) {
+  return sizeof(Plan) + held(P.sorted) + held(P.perm) + held(P.items) + held(P.mitems) + held(P.tsoff) + held(P.titems) +
+         held(P.bitems) + held(P.sitems) + held(P.objoff) + held(P.objrk) + held(P.nmodes) + held(P.gd) + held(P.gs) +
+         held(P.gout) + held(P.br);
+}
 
 t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, const int* tiles,
                     std::shared_ptr<const Plan>* out) {
@@ -546,9 +558,11 @@ t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, cons
     std::vector<int32_t> key;
     std::shared_ptr<const Plan> plan;
     uint64_t used;
+    size_t bytes;
   };
   static std::mutex mu;
   static std::vector<Entry> cache;
+  static size_t kept = 0;  // bytes of the cache
   static uint64_t clock = 0;
   bool readable = X && X->d && X->n && X->ranks && X->obj_off && X->cores && X->count >= 1 && ngroups >= 1 && gstart;
   std::vector<int32_t> key;
@@ -585,10 +599,16 @@ t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, cons
   std::shared_ptr<Plan> plan = std::make_shared<Plan>();
   T3F_CHECK(build_plan(X, ngroups, gstart, tiles, plan.get()));  // (refuses what was not readable)
   *out = plan;
+  const size_t bytes = held(key) + held(*plan);
+  if (bytes > kPlanBytes) return T3F_OK;
   std::lock_guard<std::mutex> lock(mu);
-  if (cache.size() >= kPlanCache)
-    cache.erase(std::min_element(cache.begin(), cache.end(), [](const Entry& a, const Entry& b) { return a.used < b.used; }));
-  cache.push_back(Entry{std::move(key), *out, ++clock});
+  while (cache.size() >= kPlanCache || kept + bytes > kPlanBytes) {
+    auto old = std::min_element(cache.begin(), cache.end(), [](const Entry& a, const Entry& b) { return a.used < b.used; });
+    kept -= old->bytes;
+    cache.erase(old);
+  }
+  cache.push_back(Entry{std::move(key), *out, ++clock, bytes});
+  kept += bytes;
   return T3F_OK;
 }
 
