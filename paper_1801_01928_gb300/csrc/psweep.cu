@@ -773,8 +773,10 @@ bool psweep_supported(const TTV& X, const TTV& Z) {
 static int sm_count() { return device_sm_count(); }
 
 // Objects per CTA, block shape and slices at a time. With at least four objects per SM a thread
-// takes 8 x 8 (8 x 4 fused); below that a CTA would have only a few warps, and 4 x 4 blocks with up
-// to 16 slices at a time fill it (100 objects: 1 per CTA, 256 threads instead of 64).
+// takes 8 x 8 (8 x 4 fused) if that makes four warps; else 4 x 4 blocks with up to 16 slices at a
+// time fill a CTA (100 objects: 1 per CTA, 256 threads instead of 64). Few slices leave few threads: 1000
+// objects of d = 8, r = 8, X of rank 16, project_sum and its adjoint with the larger blocks against 4 x 4, us:
+// n = 2 119, 94 -> 88, 71; n = 4 125, 105 -> 105, 86; n = 8 (X of rank 8) 146, 99 -> 125, 78.
 struct PSweepPlan {
   int J, SP;
   bool big;
@@ -791,12 +793,12 @@ static size_t psweep_smem(int RU, bool mixed, int J, int SP, int nmax) {
 static PSweepPlan plan_tiles(int RU, bool mixed, int batch, int nmax) {
   PSweepPlan p;
   int j = (batch + sm_count() - 1) / sm_count();
-  p.big = j >= 4;
-  const int G = p.big ? (RU / 8) * (mixed ? 2 : 1) : (RU / 4) * 2;
-  const int tmax = p.big ? 256 : 512;
+  p.J = j < 1 ? 1 : (j > 8 ? 8 : j);
   int np2 = 1;
   while (np2 < nmax && np2 < 16) np2 *= 2;
-  p.J = j < 1 ? 1 : (j > 8 ? 8 : j);
+  p.big = j >= 4 && p.J * np2 * (RU / 8) * (mixed ? 2 : 1) >= 128;
+  const int G = p.big ? (RU / 8) * (mixed ? 2 : 1) : (RU / 4) * 2;
+  const int tmax = p.big ? 256 : 512;
   p.SP = np2;
   while (p.SP > 1 && p.J * p.SP * G > tmax) p.SP /= 2;
   while (p.SP > 1 && psweep_smem(RU, mixed, p.J, p.SP, nmax) > 220 * 1024) p.SP /= 2;

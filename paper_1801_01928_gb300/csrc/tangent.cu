@@ -389,6 +389,18 @@ __global__ void __launch_bounds__(kThreads) k_project_core(const __grid_constant
   }
 }
 
+// Cores too small for k_project_core: one (core, object) at a time on an SM takes 4.5 to 7.5 us whatever
+// its size, while the CTAs of k_assemble_batch and k_gauge_batch share an SM and cost 0.7 us at n = 2
+// and 0.2 to 0.5 us a slice more, with r. Whole calls of 1000 rank-8 objects, d = 8, X of rank r, one kernel
+// against two, us: r = 8: n = 2 301, 105; n = 16 340, 211; r = 16: n = 4 336, 150; n = 16 404, 387; n = 30 541,
+// 720; r = 32: n = 4 394, 259; n = 8 478, 635. With few units an SM the latency of the two kernels counts:
+// 50 objects, r = 8: n = 4 49, 43; n = 8 53, 50; n = 16 53, 58; r = 16: n = 8 53, 53; r = 32: n = 4 58, 64.
+static bool small_cores(const TTV& U, int batch, int sms) {
+  long long most = 0;
+  for (int k = 0; k < U.d; ++k) most = std::max(most, U.osz[k]);
+  return (long long)U.d * batch >= 6LL * sms ? most <= 4096 : most <= 2048 && U.nmax <= 8;
+}
+
 template <int RU>
 t3f_status launch_project_core(const ProjCoreArgs& a, int sms, cudaStream_t s) {
   const size_t smem = proj_core_smem<RU>(a.mmax, a.Z.nmax);
@@ -1123,10 +1135,11 @@ extern "C" t3f_status t3f_project(const t3f_tt* U, const t3f_tt* V, const t3f_tt
   if (psweep_supported(vu, vz)) {
     int mmax = 1;
     for (int k = 0; k + 1 < vu.d; ++k) mmax = std::max(mmax, vu.r[k] * vu.n[k]);
+    const int sms = dev_sms();
     const size_t smem = vu.rmax <= 8    ? proj_core_smem<8>(mmax, vz.nmax)
                         : vu.rmax <= 16 ? proj_core_smem<16>(mmax, vz.nmax)
                                         : proj_core_smem<32>(mmax, vz.nmax);
-    if (smem <= 227 * 1024) {
+    if (smem <= 227 * 1024 && !small_cores(vu, vz.batch, sms)) {
       ProjCoreArgs p;
       memset(&p, 0, sizeof(p));
       p.U = vu;
@@ -1137,7 +1150,6 @@ extern "C" t3f_status t3f_project(const t3f_tt* U, const t3f_tt* V, const t3f_tt
       for (int j = 0; j <= vu.d; ++j) p.ioff[j] = l.ioff[j];
       p.c = c;
       p.mmax = mmax;
-      const int sms = dev_sms();
       return vu.rmax <= 8    ? launch_project_core<8>(p, sms, s)
              : vu.rmax <= 16 ? launch_project_core<16>(p, sms, s)
                              : launch_project_core<32>(p, sms, s);
