@@ -334,19 +334,24 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_bwd(const __grid_cons
 //  (1) a deterministic counting sort of the chunk's tuples by slice, for every core (warp
 //      match + per-warp prefix sums; each thread of a tuple takes every other core), giving each
 //      tuple its bucket position at core k; the next chunk's indices are fetched meanwhile;
-//  (2) both chains step core by core in bucket order, T threads each: the thread of row p at core k
-//      reads l_k (rho_{k+1}), multiplies it by its slice -- the same slice for the neighbouring
+//  (2) R = 8: both chains step core by core in bucket order, T threads each: the thread of row p at
+//      core k reads l_k (rho_{k+1}), multiplies it by its slice -- the same slice for the neighbouring
 //      rows of its bucket, so a warp reads three or four slices instead of 32 random ones -- and
-//      writes the result to its tuple's row in the order of core k + 1 (k - 1);
+//      writes the result to its tuple's row in the order of core k + 1 (k - 1). R = 4: the two threads of
+//      a tuple walk its chains through their own slices and store every partial in bucket order (a
+//      step is 16 multiply-adds, less than the barrier it would need);
 //  (3) thread per item (core k, slice s, part): a persistent R x R register accumulator
 //      adds w l_k rho_{k+1}^T over the item's share of the bucket; consecutive lanes read
 //      consecutive bucket rows.
-// No atomics in the loop; the per-CTA partial is summed in a fixed order by a second kernel.
+// The per-CTA partial is summed in a fixed order by a second kernel; the parts of a slice within one CTA
+// are summed within each warp and then by shared-memory atomics (by atomics alone, all to one address, that
+// took 35 of the 60 us of a call on 100 tuples at d = 4, n = 8, r = 8).
 // Bound by shared-memory wavefronts (a chain step reads R^2 slice values per tuple for as many
 // multiply-adds). 10^6 tuples, d = 10, n = 10, r = 8: 529 us with one thread per tuple walking both
 // chains through its own slices, 422 us with the chains on two threads (shared-memory pipe 71 %
-// busy, 5.8 wavefronts a request), now 405 us (66 %); with two sets of slices (the Riemannian form)
-// 591 -> 462 -> 452 us.
+// busy, 5.8 wavefronts a request), 405 us in bucket order (66 %); with two sets of slices (the Riemannian
+// form) 591 -> 462 -> 452 us. r = 4, 1.5 10^6 tuples: 284 us with one thread per tuple, 365 in bucket order
+// with half the tuples in flight, now 236.
 struct CompletionArgs {
   GatherArgs g;
   int T;                      // tuples per chunk (half of blockDim.x)
@@ -420,6 +425,7 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
   for (int a = 0; a < R; ++a)
 #pragma unroll
     for (int b = 0; b < R; ++b) acc[a][b] = 0.0f;
+  bool used = false;  // the item has had a tuple
   double lsum = 0.0;
   __syncthreads();
 
@@ -478,30 +484,30 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
       }
     }
     __syncthreads();
-    for (int k = grp; k < d; k += 2) {
-      const int sl = IDX[k * T + tt], p = WC[(k * NB + sl) * NW + tw] + POS[k * T + tt];
-      POS[k * T + tt] = (unsigned char)p;
-      TID[k * T + p] = (unsigned char)tt;
-      SLC[k * T + p] = (unsigned char)sl;
-    }
-    __syncthreads();
-    // (2) the chains, row tt of each core in turn
-    for (int q = 0; q + 1 < d; ++q) {
-      if (tt < nv) {
+    if constexpr (R == 4) {
+      // (2) the tuple's chains; p = its row in the bucket order of core k
+      if (valid) {
+        float v[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) v[a] = a == 0 ? 1.0f : 0.0f;
         if (grp == 0) {
-          const int k = d - 1 - q;
-          const float* S = Rs + (k * nmax + SLC[k * T + tt]) * SS;
-          const int p = POS[(k - 1) * T + TID[k * T + tt]];
-          float v[R], nr[R];
-          if (q == 0) {
+          for (int k = d - 1; k >= 0; --k) {
+            const int sl = IDX[k * T + tt];
+            const float* S = Rs + (k * nmax + sl) * SS;
+            if (k < d - 1) {
+              const int p = WC[(k * NB + sl) * NW + tw] + POS[k * T + tt];
 #pragma unroll
-            for (int a = 0; a < R; ++a) nr[a] = S[a * R];
-          } else {
-#pragma unroll
-            for (int h = 0; h < H; ++h) {
-              const float4 r4 = RH[((size_t)k * H + h) * T + tt];
-              v[4 * h] = r4.x; v[4 * h + 1] = r4.y; v[4 * h + 2] = r4.z; v[4 * h + 3] = r4.w;
+              for (int h = 0; h < H; ++h)
+                RH[((size_t)k * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
             }
+            if (k == 0) {
+              float x = 0.0f;
+#pragma unroll
+              for (int b = 0; b < R; ++b) x = fmaf(S[b], v[b], x);
+              v[0] = x;
+              break;
+            }
+            float nr[R];
 #pragma unroll
             for (int a = 0; a < R; ++a) {
               float acc1 = 0.0f;
@@ -515,24 +521,28 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
               }
               nr[a] = acc1;
             }
+#pragma unroll
+            for (int a = 0; a < R; ++a) v[a] = nr[a];
           }
-#pragma unroll
-          for (int h = 0; h < H; ++h)
-            RH[((size_t)(k - 1) * H + h) * T + p] = make_float4(nr[4 * h], nr[4 * h + 1], nr[4 * h + 2], nr[4 * h + 3]);
+          float wt = yt;
+          if (!g.w) {
+            const double res = (double)v[0] - (double)yt;
+            lsum += 0.5 * res * res;
+            wt = (float)res;
+          }
+          Wt[tt] = wt;
         } else {
-          const int k = q;
-          const float* S = Ls + (k * nmax + SLC[k * T + tt]) * SS;
-          const int p = POS[(k + 1) * T + TID[k * T + tt]];
-          float v[R], nl[R];
-          if (q == 0) {
+          for (int k = 0; k < d; ++k) {
+            const int sl = IDX[k * T + tt];
+            const int p = WC[(k * NB + sl) * NW + tw] + POS[k * T + tt];
+            TID[k * T + p] = (unsigned char)tt;
+            if (k > 0)
 #pragma unroll
-            for (int b = 0; b < R; ++b) nl[b] = S[b];
-          } else {
-#pragma unroll
-            for (int h = 0; h < H; ++h) {
-              const float4 l4 = LW[((size_t)(k - 1) * H + h) * T + tt];
-              v[4 * h] = l4.x; v[4 * h + 1] = l4.y; v[4 * h + 2] = l4.z; v[4 * h + 3] = l4.w;
-            }
+              for (int h = 0; h < H; ++h)
+                LW[((size_t)(k - 1) * H + h) * T + p] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+            if (k + 1 == d) break;
+            const float* S = Ls + (k * nmax + sl) * SS;
+            float nl[R];
 #pragma unroll
             for (int b = 0; b < R; ++b) nl[b] = 0.0f;
 #pragma unroll
@@ -546,35 +556,110 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
                 nl[b + 3] = fmaf(v[a], s4.w, nl[b + 3]);
               }
             }
-          }
 #pragma unroll
-          for (int h = 0; h < H; ++h)
-            LW[((size_t)k * H + h) * T + p] = make_float4(nl[4 * h], nl[4 * h + 1], nl[4 * h + 2], nl[4 * h + 3]);
+            for (int b = 0; b < R; ++b) v[b] = nl[b];
+          }
         }
+      }
+    } else {
+      for (int k = grp; k < d; k += 2) {
+        const int sl = IDX[k * T + tt], p = WC[(k * NB + sl) * NW + tw] + POS[k * T + tt];
+        POS[k * T + tt] = (unsigned char)p;
+        TID[k * T + p] = (unsigned char)tt;
+        SLC[k * T + p] = (unsigned char)sl;
       }
       __syncthreads();
-    }
-    // the value (from the suffix cores), residual and weight of row tt of the first core
-    if (grp == 0 && tt < nv) {
-      const float* S = Rs + SLC[tt] * SS;
-      const int o = TID[tt];
-      float x = S[0];
-      if (d > 1) {
-        x = 0.0f;
+      // (2) the chains, row tt of each core in turn
+      for (int q = 0; q + 1 < d; ++q) {
+        if (tt < nv) {
+          if (grp == 0) {
+            const int k = d - 1 - q;
+            const float* S = Rs + (k * nmax + SLC[k * T + tt]) * SS;
+            const int p = POS[(k - 1) * T + TID[k * T + tt]];
+            float v[R], nr[R];
+            if (q == 0) {
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const float4 r4 = RH[(size_t)h * T + tt];
-          const float4 s4 = *reinterpret_cast<const float4*>(S + 4 * h);
-          x = fmaf(s4.x, r4.x, x);
-          x = fmaf(s4.y, r4.y, x);
-          x = fmaf(s4.z, r4.z, x);
-          x = fmaf(s4.w, r4.w, x);
+              for (int a = 0; a < R; ++a) nr[a] = S[a * R];
+            } else {
+#pragma unroll
+              for (int h = 0; h < H; ++h) {
+                const float4 r4 = RH[((size_t)k * H + h) * T + tt];
+                v[4 * h] = r4.x; v[4 * h + 1] = r4.y; v[4 * h + 2] = r4.z; v[4 * h + 3] = r4.w;
+              }
+#pragma unroll
+              for (int a = 0; a < R; ++a) {
+                float acc1 = 0.0f;
+#pragma unroll
+                for (int b = 0; b < R; b += 4) {
+                  const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+                  acc1 = fmaf(s4.x, v[b], acc1);
+                  acc1 = fmaf(s4.y, v[b + 1], acc1);
+                  acc1 = fmaf(s4.z, v[b + 2], acc1);
+                  acc1 = fmaf(s4.w, v[b + 3], acc1);
+                }
+                nr[a] = acc1;
+              }
+            }
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+              RH[((size_t)(k - 1) * H + h) * T + p] = make_float4(nr[4 * h], nr[4 * h + 1], nr[4 * h + 2], nr[4 * h + 3]);
+          } else {
+            const int k = q;
+            const float* S = Ls + (k * nmax + SLC[k * T + tt]) * SS;
+            const int p = POS[(k + 1) * T + TID[k * T + tt]];
+            float v[R], nl[R];
+            if (q == 0) {
+#pragma unroll
+              for (int b = 0; b < R; ++b) nl[b] = S[b];
+            } else {
+#pragma unroll
+              for (int h = 0; h < H; ++h) {
+                const float4 l4 = LW[((size_t)(k - 1) * H + h) * T + tt];
+                v[4 * h] = l4.x; v[4 * h + 1] = l4.y; v[4 * h + 2] = l4.z; v[4 * h + 3] = l4.w;
+              }
+#pragma unroll
+              for (int b = 0; b < R; ++b) nl[b] = 0.0f;
+#pragma unroll
+              for (int a = 0; a < R; ++a) {
+#pragma unroll
+                for (int b = 0; b < R; b += 4) {
+                  const float4 s4 = *reinterpret_cast<const float4*>(S + a * R + b);
+                  nl[b] = fmaf(v[a], s4.x, nl[b]);
+                  nl[b + 1] = fmaf(v[a], s4.y, nl[b + 1]);
+                  nl[b + 2] = fmaf(v[a], s4.z, nl[b + 2]);
+                  nl[b + 3] = fmaf(v[a], s4.w, nl[b + 3]);
+                }
+              }
+            }
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+              LW[((size_t)k * H + h) * T + p] = make_float4(nl[4 * h], nl[4 * h + 1], nl[4 * h + 2], nl[4 * h + 3]);
+          }
         }
+        __syncthreads();
       }
-      if (!g.w) {
-        const double res = (double)x - (double)Wt[o];
-        lsum += 0.5 * res * res;
-        Wt[o] = (float)res;
+      // the value (from the suffix cores), residual and weight of row tt of the first core
+      if (grp == 0 && tt < nv) {
+        const float* S = Rs + SLC[tt] * SS;
+        const int o = TID[tt];
+        float x = S[0];
+        if (d > 1) {
+          x = 0.0f;
+#pragma unroll
+          for (int h = 0; h < H; ++h) {
+            const float4 r4 = RH[(size_t)h * T + tt];
+            const float4 s4 = *reinterpret_cast<const float4*>(S + 4 * h);
+            x = fmaf(s4.x, r4.x, x);
+            x = fmaf(s4.y, r4.y, x);
+            x = fmaf(s4.z, r4.z, x);
+            x = fmaf(s4.w, r4.w, x);
+          }
+        }
+        if (!g.w) {
+          const double res = (double)x - (double)Wt[o];
+          lsum += 0.5 * res * res;
+          Wt[o] = (float)res;
+        }
       }
     }
     __syncthreads();
@@ -582,6 +667,7 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
     // core, rho = 1 after the last)
     if (ik >= 0) {
       const int p0 = BO[ik * NB + is], p1 = BO[ik * NB + is + 1];
+      used = used || p0 + ip < p1;
       const unsigned char* tb = TID + (size_t)ik * T;
       const float4* lw = LW + (size_t)(ik - 1) * H * T;
       const float4* rh = RH + (size_t)ik * H * T;
@@ -638,13 +724,31 @@ __global__ void __launch_bounds__(512) k_completion(const __grid_constant__ Comp
   float* cacc = reinterpret_cast<float*>(RH);  // d * nmax * R * R floats (fits the region)
   for (int e = tid; e < d * nmax * R * R; e += blockDim.x) cacc[e] = 0.0f;
   __syncthreads();
-  if (ik >= 0) {
-    float* dst = cacc + (ik * nmax + is) * R * R;
+  if (const int lanes = __popc(__ballot_sync(0xffffffffu, used))) {
+    // the parts of a slice sit on neighbouring lanes: their sum within the warp ends in the lane of the first
+    // (a warp with a few tuples adds them directly)
+    const int left = ik < 0 ? 1 : np - ip;  // lanes of this slice from here on
+    int most = 1;
+    if (lanes > 4)
+      for (int k = 0; k < d; ++k) most = max(most, min(ca.parts[k], 32));
+    for (int o = 1; o < most; o <<= 1) {
+      const bool on = o < left && lane + o < 32;
 #pragma unroll
-    for (int a = 0; a < R; ++a)
+      for (int a = 0; a < R; ++a)
 #pragma unroll
-      for (int b = 0; b < R; ++b)
-        if (acc[a][b] != 0.0f) atomicAdd(dst + a * R + b, acc[a][b]);
+        for (int b = 0; b < R; ++b) {
+          const float v = __shfl_down_sync(0xffffffffu, acc[a][b], o);
+          if (on) acc[a][b] += v;
+        }
+    }
+    if (ik >= 0 && (most == 1 || lane == 0 || ip == 0)) {
+      float* dst = cacc + (ik * nmax + is) * R * R;
+#pragma unroll
+      for (int a = 0; a < R; ++a)
+#pragma unroll
+        for (int b = 0; b < R; ++b)
+          if (acc[a][b] != 0.0f) atomicAdd(dst + a * R + b, acc[a][b]);
+    }
   }
   __syncthreads();
   float* out = g.grad_part + (long long)blockIdx.x * g.gsize;
@@ -758,8 +862,11 @@ static size_t completion_smem(const TTV& L, const TTV& Rv, int R, int T, bool sa
 }
 
 // Choose the bucketed adjoint when its items fit one CTA and its buffers fit shared memory: the
-// largest chunk T <= 256 of one CTA per SM, or the largest of two CTAs per SM (one CTA's barrier
-// waits overlap the other's chains) where that keeps three quarters of its tuples in flight.
+// largest chunk T <= 256 of one CTA per SM, or the largest of two (one CTA's barrier waits overlap the
+// other's chains; up to 256 threads at the 128 registers of R = 8, 512 at the 64 of R = 4) where that keeps
+// as many tuples in flight, or for R = 4 of four on the same condition. 1.5 10^6 tuples, r = 4: d = 10, n = 10
+// two CTAs of 256 tuples 252 us, four of 128 236; d = 30, n = 4 two CTAs of fewer tuples than one holds
+// 1255 us, one 986.
 static bool plan_completion(const TTV& L, const TTV& Rv, bool same, int R, GatherLayout* lay) {
   if (R > 8 || L.nmax > 254) return false;
   const int d = L.d;
@@ -769,19 +876,17 @@ static bool plan_completion(const TTV& L, const TTV& Rv, bool same, int R, Gathe
     if (k == 0 || k == d - 1) bnd += L.n[k];
     else inner += L.n[k];
   }
-  auto best = [&](size_t cap) {
-    for (int T = 256; T >= 64; T -= 32) {
-      if (completion_smem(L, Rv, R, T, same) > cap || bnd + inner > 2 * T) continue;
-      return T;
-    }
+  // the largest chunk of at most `most` tuples that leaves room for `ctas` CTAs on an SM, 0 where none does
+  auto best = [&](int ctas, int most) {
+    const size_t cap = ctas == 1 ? 220 * 1024 : (228 * 1024 - ctas * 1400) / ctas;
+    for (int T = most; T >= 64; T -= 32)
+      if (completion_smem(L, Rv, R, T, same) <= cap && bnd + inner <= 2 * T) return T;
     return 0;
   };
-  // two CTAs per SM: 228 KB per SM less 1 KB reserved and the static block per CTA; 128 registers a
-  // thread leave room for two CTAs of up to 256 threads
-  const int T1 = best(220 * 1024), T2 = std::min(128, best((228 * 1024 - 2 * 1400) / 2));
+  const int T1 = best(1, 256), T2 = best(2, R == 4 ? 256 : 128), T4 = R == 4 ? best(4, 128) : 0;
   if (!T1) return false;
-  const bool two = T2 > 0 && bnd + inner <= 2 * T2 && 8 * T2 >= 3 * T1;
-  const int T = two ? T2 : T1;
+  const bool two = T2 > 0 && 2 * T2 >= T1, four = two && T4 > 0 && 2 * T4 >= T2;
+  const int T = four ? T4 : two ? T2 : T1;
   const int P2 = inner ? (2 * T - bnd) / inner : 1;
   int it = 0;
   for (int k = 0; k < d; ++k) {
@@ -790,7 +895,7 @@ static bool plan_completion(const TTV& L, const TTV& Rv, bool same, int R, Gathe
     it += L.n[k] * lay->parts[k];
   }
   lay->item0[d] = it;
-  lay->bucketed = two ? 2 : 1;  // CTAs per SM
+  lay->bucketed = four ? 4 : two ? 2 : 1;  // CTAs per SM
   lay->T = T;
   lay->NB = L.nmax + 1;
   lay->region = (int)completion_region(L, Rv, R, T, same);
