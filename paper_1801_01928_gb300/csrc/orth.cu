@@ -17,7 +17,7 @@
 // alternate between two buffers). R is then broadcast to every CTA and Q = W R^{-1} is
 // recovered row by row by a triangular solve that needs no further communication.
 //
-// Tall unfoldings of at most 32 columns first try a factorisation with two exchanges instead of
+// Tall unfoldings of 4 to 32 columns first try a factorisation with two exchanges instead of
 // one per column (cqr_step): a Cholesky factor R1 of the Gram matrix taken in FP32 preconditions
 // W, Q1 = W R1^{-1} in FP64 is orthonormal to some 1e-6, and one FP64 Gram matrix of Q1 corrects
 // both factors to FP64 accuracy. The departure of Q1 from orthonormality is measured; where it
@@ -25,7 +25,9 @@
 // config 5 (d = 20, n = 16, r = 32, 57 factorisations): 6.80 ms with Householder columns alone (3.3
 // us each: one cluster barrier, four block barriers and the FP64 chain of the reflector), 2.53 ms
 // now, 40 us a factorisation, of which the 2.3 thousand FP64 warp instructions of a CTA's 32 rows
-// at some 16 clocks each are 18 us.
+// at some 16 clocks each are 18 us. The left-to-right and the last sweep factor unfoldings that carry the
+// singular values of X; with sigma_1 / sigma_r = 100, 300 and 1000 or more at every interface the same size
+// takes 3.07, 3.37 and 4.45 ms (the refused steps pay for both ways), with Householder columns alone 6.90.
 //
 // The working cores keep their original row strides so every in-place update touches only the
 // rows or columns its CTA owns.
@@ -556,9 +558,18 @@ __device__ void householder_step(const OrthArgs& a, const double* core, const Di
 
 // out(a, x) = sum_{al >= a} R(a, al) in(al, x) for a < kk, x < nx: the lanes of a warp run over x with
 // one row a (sums of equal length), and a thread takes the rows a and kk - 1 - a together, so every
-// thread does the same work on two independent chains.
+// thread does the same work on two independent chains (up to three rows: one element a thread).
 template <class FR, class FI, class FO>
 __device__ __forceinline__ void push_rows(int kk, int c, int nx, FR R, FI in, FO out) {
+  if (kk < 4) {
+    for (int e = threadIdx.x; e < kk * nx; e += blockDim.x) {
+      const int a = e / nx, x = e % nx;
+      double u = 0.0;
+      for (int al = a; al < c; ++al) u = fma(R(a, al), in(al, x), u);
+      out(a, x, u);
+    }
+    return;
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int na = (kk + 1) / 2, ng = (nx + 31) / 32;
   for (int w = warp; w < na * ng; w += nw) {
@@ -600,8 +611,12 @@ __device__ void qr_step(const OrthArgs& a, double* base, Dims* dims, int k, int 
   }
   __syncthreads();
 
+  // A Householder column is 2.5 to 3.5 us, cqr_step some 12 to 15 us up to eight columns, and a square
+  // unfolding is often refused. d = 8, n = 8, Householder against cqr_step, us: r = 1 148, 229; r = 2 222, 261;
+  // r = 3 283, 269; r = 4 338, 280; r = 5 394, 286; d = 10, n = 4: r = 3 361, 342; 4 x 4 and 4 x 5 unfoldings
+  // (d = 2, n = 4) 52, 58.
   bool done = false;
-  if (c <= kCqrMax && m >= c) {
+  if (c >= 4 && c <= kCqrMax && m >= (c < 6 ? c + 1 : c)) {
     done = cqr_step(a, s, nrow, c, cluster);
     if (!done) {  // the rows again, for the Householder columns
       __syncthreads();
