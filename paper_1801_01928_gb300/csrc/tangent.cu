@@ -1203,7 +1203,11 @@ extern "C" t3f_status t3f_tangent_gram(const t3f_tt* dA, const t3f_tt* dB, float
   g.part = reinterpret_cast<float*>(static_cast<char*>(ws) + p.part_off);
   const long long grid = (long long)p.tilesA * p.tilesB * p.nsplit;
   if (grid > 0x7fffffffLL) return T3F_ERR_UNSUPPORTED;
-  if (g.self && p.tilesA == 1) {  // one tile of a self Gram matrix: its upper triangle
+  // One tile of a self Gram matrix: its upper triangle, where the coordinates (nchunks x 16) outweigh the
+  // sum over the teams at the end. Batch 25, triangle against tile, us: 2 10^2 coordinates 22.7, 12.4; 3.2 10^3
+  // 28.8, 26.8; 5.3 10^3 28.8, 28.8; 5 10^4 37, 66; 2.9 10^5 82, 268. From 121 vectors on one team does all:
+  // 128 vectors and 2 10^4 coordinates 37, 31; 7 10^4 72, 70; 10^5 92, 94; 2.9 10^5 249, 274.
+  if (g.self && p.tilesA == 1 && p.nchunks >= 320 && (va.batch <= 120 || p.cper >= 20)) {
     TGramSymArgs y;
     memset(&y, 0, sizeof(y));
     y.g = g;
