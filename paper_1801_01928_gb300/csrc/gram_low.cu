@@ -15,7 +15,8 @@
 //   row role     R' += X B_i^T,  Y = R B_i^T,  dA_a,i = sum_b (g M) Y^T
 // a lane sums dB (dA) over its objects, the S sub-objects meet by shuffles and one atomic per
 // element and tile goes to the gradient. The left partials of every interface go through a scratch
-// area per tile (t R x t RP floats each, a full batch's no more than the 4 x 4 block kernels').
+// area per tile (t R x t RP floats each, R of the larger rank on both sides: as much as the 4 x 4 block
+// kernels' on equal sides, ranks 6 and 4 48 floats a pair and interface instead of 32).
 //
 // 100 x 100 pairs, d = 10, n = 10, r = 10: forward 388 us with 4 x 4 blocks on padded ranks (three
 // barriers per slice) -> 203 us, adjoint 1826 -> 783 us. Bound by the issue of the two or three warps a
@@ -48,6 +49,7 @@ struct Low {
 struct GramLowArgs {
   TTV A, B;
   int t;                 // objects a side of a tile
+  int cut;               // forward: padded ranks run with the row test
   float* out;            // forward
   const float* dG;       // adjoint
   float* dA;
@@ -162,9 +164,9 @@ struct LowSlices {
 enum { kCut, kPadded, kExact };
 
 template <int R, class F>
-__device__ __forceinline__ void by_ranks(int lo, F f) {
+__device__ __forceinline__ void by_ranks(int lo, bool cut, F f) {
   if (lo == R) f(std::integral_constant<int, kExact>());
-  else if (((lo + 3) & ~3) >= R) f(std::integral_constant<int, kPadded>());
+  else if (((lo + 3) & ~3) >= R && !cut) f(std::integral_constant<int, kPadded>());
   else f(std::integral_constant<int, kCut>());
 }
 template <int MODE>
@@ -260,7 +262,7 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
           }
       }
     };
-    by_ranks<R>(min(eA0, eB0), slices);
+    by_ranks<R>(min(eA0, eB0), g.cut, slices);
     if (k + 1 == kend && !SAVE) break;
     // the columns of M' become the rows of the next core's M
     if (on && w < nb)
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(32 * Low<R>::W, Low<R>::W <= 8 ? 2 : 1) k_gram
         }
       }
     };
-    by_ranks<R>(min(min(eA0, eA1), min(eB0, eB1)), slices);
+    by_ranks<R>(min(min(eA0, eA1), min(eB0, eB1)), false, slices);
     if (k == 0) break;
     // R' : rows to columns through the X buffer that the last slice did not use
     float* Rs = Xs + (c & 1) * L::MAT;
@@ -520,13 +522,17 @@ auto low_dispatch(const TTV& A, const TTV& B, F f) {
 // file against the 4 x 4 block kernels; n modes a core, d cores):
 //   largest rank 1 .. 10, the sides within a half of one another (a side of 6 against 10 gains
 //   nothing at all; up to rank 4 every pair of ranks): forward 34 .. 208 against 90 .. 401 and adjoint
-//   92 .. 821 against 250 .. 1856 over batches of 8 x 9 .. 128 x 128, 1.1 to 4.2 times as fast;
-//   11 and 12, forward only and up to 64 pairs an SM: 80 x 80 116 against 154, but 128 x 128 with n = 16,
-//   d = 4 311 against 290 (two objects of 12 rows a warp); the adjoint 966 against 927 at 96 x 104;
-//   13 .. 16, both sides: forward 92 .. 802 against 283 .. 1068. The adjoint's three sets of rows
-//   take all registers, 551 against 424 on 8 x 9 pairs and 952 against 789 on 25 x 56, but 552
-//   against 919 on 64 x 64 and 2487 against 3304 on 128 x 128, so from 4096 pairs on, and only where no inner
-//   core is of much lower rank (1-4-16-16-16-4-1, 100 x 100: 790 against 727).
+//   92 .. 821 against 250 .. 1856 over batches of 8 x 9 .. 128 x 128, 1.1 to 4.2 times as fast. Forward of
+//   many pairs of ranks 1 and 2 (d = 10, n = 10): 200 x 200 115 against 148, 350 x 350 247 against 225, 500 x
+//   500 445 against 421, 800 x 800 1062 against 1198, so not from 500 to 3000 pairs an SM;
+//   11 and 12, forward only and up to 46 pairs an SM: 80 x 80 138 against 172, but 90 x 90 of ranks 12 and 9 177
+//   against 168, 128 x 128 with n = 16, d = 4 311 against 290 (two objects of 12 rows a warp); the adjoint 966
+//   against 927 at 96 x 104;
+//   13 .. 16, both sides: forward 92 .. 802 against 283 .. 1068, except many pairs whose inner cores are of
+//   lower rank (61 x 304 of ranks 1 to 15 727 against 619; 24 x 5 of ranks 3 to 16 148 against 294). The
+//   adjoint's three sets of rows take all registers, 551 against 424 on 8 x 9 pairs and 952 against 789 on
+//   25 x 56, but 552 against 919 on 64 x 64 and 2487 against 3304 on 128 x 128, so from 4096 pairs on, and
+//   only where no inner core is of much lower rank (1-4-16-16-16-4-1, 100 x 100: 790 against 727).
 static bool low_ranks(const TTV& A, const TTV& B) {
   const int hi = std::max(A.rmax, B.rmax), lo = std::min(A.rmax, B.rmax);
   if (A.dtype != T3F_F32 || B.dtype != T3F_F32 || hi > 16) return false;
@@ -536,18 +542,28 @@ static bool low_ranks(const TTV& A, const TTV& B) {
   return hi <= 10 ? 3 * lo >= 2 * hi : ((lo + 3) & ~3) >= hi;
 }
 
+// Every inner core of the ranks that only R = 14 and 16 hold.
+static bool inner_full(const TTV& A, const TTV& B) {
+  for (int k = 1; k < A.d; ++k)
+    if (std::min(A.r[k], B.r[k]) <= 12) return false;
+  return true;
+}
+
 bool gram_low_supported(const TTV& A, const TTV& B) {
+  if (!low_ranks(A, B)) return false;
   const int hi = std::max(A.rmax, B.rmax);
-  return low_ranks(A, B) && (hi <= 10 || hi > 12 || (long long)A.batch * B.batch <= 64LL * device_sm_count());
+  const long long pairs = (long long)A.batch * B.batch, sms = device_sm_count();
+  if (hi <= 2) return pairs <= 500 * sms || pairs >= 3000 * sms;
+  if (hi <= 10) return true;
+  if (hi <= 12) return pairs <= 46 * sms;
+  return pairs <= 64 * sms || inner_full(A, B);
 }
 
 bool gram_low_bwd_supported(const TTV& A, const TTV& B) {
   if (!low_ranks(A, B)) return false;
-  if (std::max(A.rmax, B.rmax) <= 10) return true;
-  if ((long long)A.batch * B.batch < 4096) return false;
-  for (int k = 1; k < A.d; ++k)
-    if (std::min(A.r[k], B.r[k]) <= 12) return false;
-  return true;
+  const int hi = std::max(A.rmax, B.rmax);
+  if (hi <= 10) return true;
+  return hi > 12 && (long long)A.batch * B.batch >= 4096 && inner_full(A, B);
 }
 
 size_t ws_gram_low_bwd(const TTV& A, const TTV& B) {
@@ -562,6 +578,9 @@ size_t ws_gram_low_bwd(const TTV& A, const TTV& B) {
 template <int R, class K>
 static t3f_status launch_low(K kern, GramLowArgs& g, cudaStream_t s) {
   g.t = low_tile<R>(g.A, g.B);
+  // Many pairs of ranks 1 to 3 (R = 4): the additions for padding count, not the loads' latency (padded
+  // against cut, ranks 2, d = 10, n = 10, us: 100 x 100 47.6, 49.7; 200 x 200 123, 115; 500 x 500 538, 445).
+  g.cut = R == 4 && (long long)g.A.batch * g.B.batch > 150LL * device_sm_count();
   const long long tiles = (long long)((g.A.batch + g.t - 1) / g.t) * ((g.B.batch + g.t - 1) / g.t);
   if (tiles > 0x7fffffff) return T3F_ERR_UNSUPPORTED;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Low<R>::smem) != cudaSuccess)
@@ -595,7 +614,7 @@ t3f_status run_gram_low_bwd(const TTV& A, const TTV& B, const float* dG, float* 
   g.scratch = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
   return low_dispatch(A, B, [&](auto rc) -> t3f_status {
     constexpr int R = decltype(rc)::value;
-    if constexpr (R == 12) return T3F_ERR_UNSUPPORTED;  // never taken by the rule above
+    if constexpr (R == 12) return T3F_ERR_UNSUPPORTED;  // (gram_low_bwd_supported takes no rank of 11 or 12)
     else return launch_low<R>(k_gram_low_bwd<R>, g, s);
   });
 }
