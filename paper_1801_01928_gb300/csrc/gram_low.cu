@@ -288,8 +288,10 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
+// Two blocks an SM at R = 4 (64 registers, for large batches) and R = 8 (128), one elsewhere: left to the
+// compiler, R = 8 had 80 registers (100 x 100 pairs of rank 7, d = 6, n = 10: 95 us, now 80) and R = 16 168 (471, now 408).
 template <int R>
-__global__ void __launch_bounds__(32 * Low<R>::W) k_gram_low(const __grid_constant__ GramLowArgs g) {
+__global__ void __launch_bounds__(32 * Low<R>::W, R == 4 || R == 8 ? 2 : 1) k_gram_low(const __grid_constant__ GramLowArgs g) {
   extern __shared__ __align__(16) float sm[];
   const int ntb = (g.B.batch + g.t - 1) / g.t;
   const int a0 = (blockIdx.x / ntb) * g.t, b0 = (blockIdx.x % ntb) * g.t;
