@@ -25,6 +25,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "t3f_internal.cuh"
 
@@ -83,12 +84,15 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // y0, y1 <- (I - tau v v^T) y0, y1 with the vectors spread over the lanes (element 32 c + lane
-// in slot c); the slots below c0 hold zeros of v.
-__device__ __forceinline__ void reflect2(const double (&v)[kRegRows], double tau, int c0, int nch,
-                                         double (&y0)[kRegRows], double (&y1)[kRegRows]) {
+// in slot c); the slots below c0 hold zeros of v. NC: the slots a column of this height can use, at
+// compile time, since an FP64 instruction that is predicated off takes its turn on the pipe all the same
+// (16 slots for every height: 21 objects of rank 46, d = 8, n = 2, to rank 12 2970 us, now 1390).
+template <int NC>
+__device__ __forceinline__ void reflect2(const double (&v)[NC], double tau, int c0, int nch, double (&y0)[NC],
+                                         double (&y1)[NC]) {
   double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c)
+  for (int c = 0; c < NC; ++c)
     if (c >= c0 && c < nch) {
       s0 = fma(v[c], y0[c], s0);
       s1 = fma(v[c], y1[c], s1);
@@ -97,42 +101,144 @@ __device__ __forceinline__ void reflect2(const double (&v)[kRegRows], double tau
   s0 *= -tau;
   s1 *= -tau;
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c)
+  for (int c = 0; c < NC; ++c)
     if (c >= c0 && c < nch) {
       y0[c] = fma(s0, v[c], y0[c]);
       y1[c] = fma(s1, v[c], y1[c]);
     }
 }
 
-__device__ __forceinline__ void reflect1(const double (&v)[kRegRows], double tau, int c0, int nch,
-                                         double (&y)[kRegRows]) {
+template <int NC>
+__device__ __forceinline__ void reflect1(const double (&v)[NC], double tau, int c0, int nch, double (&y)[NC]) {
   double s0 = 0.0, s1 = 0.0;  // two chains: one column alone is latency-bound
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c)
+  for (int c = 0; c < NC; ++c)
     if (c >= c0 && c < nch) {
       if (c & 1) s1 = fma(v[c], y[c], s1);
       else s0 = fma(v[c], y[c], s0);
     }
   const double s = -tau * warp_sum(s0 + s1);
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c)
+  for (int c = 0; c < NC; ++c)
     if (c >= c0 && c < nch) y[c] = fma(s, v[c], y[c]);
 }
 
-__device__ __forceinline__ void load_col(const double* p, int m, int nch, double (&y)[kRegRows]) {
+template <int NC>
+__device__ __forceinline__ void load_col(const double* p, int m, int nch, double (&y)[NC]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c) {
+  for (int c = 0; c < NC; ++c) {
     y[c] = 0.0;
     if (c < nch && 32 * c + lane < m) y[c] = p[32 * c + lane];
   }
 }
 
-__device__ __forceinline__ void store_col(double* p, int m, int nch, const double (&y)[kRegRows]) {
+template <int NC>
+__device__ __forceinline__ void store_col(double* p, int m, int nch, const double (&y)[NC]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int c = 0; c < kRegRows; ++c)
+  for (int c = 0; c < NC; ++c)
     if (c < nch && 32 * c + lane < m) p[32 * c + lane] = y[c];
+}
+
+// f with the register slots of a column of m <= 32 kRegRows rows.
+template <class F>
+__device__ __forceinline__ void by_slots(int m, F f) {
+  if (m <= 32) f(std::integral_constant<int, 1>());
+  else if (m <= 64) f(std::integral_constant<int, 2>());
+  else if (m <= 128) f(std::integral_constant<int, 4>());
+  else if (m <= 256) f(std::integral_constant<int, 8>());
+  else f(std::integral_constant<int, kRegRows>());
+}
+
+// The QR below for columns of at most 32 NC rows, panel by panel.
+template <int NC>
+__device__ void qr_panels(double* A, int m, int c, double* vp, double* tp) {
+  const int q = min(m, c);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kRoundThreads / 32;
+  const int nch = (m + 31) / 32;
+  for (int j0 = 0; j0 < q; j0 += kPanel) {
+    const int nb = min(kPanel, q - j0), cb = j0 / 32;
+    {  // factor the panel: warp w holds column j0 + w
+      double y[NC];
+      const bool mine = warp < nb;
+      if (mine) load_col(A + (long long)(j0 + warp) * m, m, nch, y);
+      for (int jj = 0; jj < nb; ++jj) {
+        const int j = j0 + jj;
+        double* vj = vp + jj * (32 * NC);
+        if (warp == jj) {
+          double part = 0.0, x0 = 0.0;
+#pragma unroll
+          for (int c2 = 0; c2 < NC; ++c2)
+            if (c2 >= cb && c2 < nch) {
+              const int i = 32 * c2 + lane;
+              if (i >= j) part = fma(y[c2], y[c2], part);
+              if (i == j) x0 = y[c2];
+            }
+          part = warp_sum(part);
+          x0 = __shfl_sync(0xffffffffu, x0, j & 31);
+          double alpha = 0.0, tau = 0.0, inv = 0.0;
+          if (part > 0.0) {
+            const double rn = rsqrt(part);
+            alpha = x0 >= 0.0 ? -(part * rn) : part * rn;
+            tau = fma(fabs(x0), rn, 1.0);  // -v0 / alpha
+            inv = 1.0 / (x0 - alpha);
+          }
+#pragma unroll
+          for (int c2 = 0; c2 < NC; ++c2)
+            if (c2 < nch) {
+              const int i = 32 * c2 + lane;
+              if (i >= j) y[c2] = i == j ? alpha : y[c2] * inv;
+              vj[i] = i > j ? y[c2] : (i == j ? 1.0 : 0.0);
+            }
+          if (lane == 0) tp[jj] = tau;
+        }
+        __syncthreads();
+        if (mine && warp > jj) {
+          double s = 0.0;
+#pragma unroll
+          for (int c2 = 0; c2 < NC; ++c2)
+            if (c2 >= cb && c2 < nch) s = fma(vj[32 * c2 + lane], y[c2], s);
+          s = -tp[jj] * warp_sum(s);
+#pragma unroll
+          for (int c2 = 0; c2 < NC; ++c2)
+            if (c2 >= cb && c2 < nch) y[c2] = fma(s, vj[32 * c2 + lane], y[c2]);
+        }
+      }
+      if (mine) store_col(A + (long long)(j0 + warp) * m, m, nch, y);
+    }
+    // the panel's reflectors over the trailing columns, two per warp at a time (one per warp when
+    // at most eight are left, so that the last round spreads over all warps)
+    for (int l0 = j0 + nb; l0 < c; l0 += 2 * nw) {
+      const bool pairs = c - l0 > nw;
+      const int l = l0 + (pairs ? 2 * warp : warp);
+      if (l >= c) break;
+      double y0[NC], y1[NC], v[NC];
+      const bool two = pairs && l + 1 < c;
+      if (!two) {
+        load_col(A + (long long)l * m, m, nch, y0);
+        for (int jj = 0; jj < nb; ++jj) {
+          const double* vj = vp + jj * (32 * NC);
+#pragma unroll
+          for (int c2 = 0; c2 < NC; ++c2) v[c2] = c2 >= cb && c2 < nch ? vj[32 * c2 + lane] : 0.0;
+          reflect1(v, tp[jj], cb, nch, y0);
+        }
+        store_col(A + (long long)l * m, m, nch, y0);
+        continue;
+      }
+      load_col(A + (long long)l * m, m, nch, y0);
+      load_col(A + (long long)(l + 1) * m, m, nch, y1);
+      for (int jj = 0; jj < nb; ++jj) {
+        const double* vj = vp + jj * (32 * NC);
+#pragma unroll
+        for (int c2 = 0; c2 < NC; ++c2) v[c2] = c2 >= cb && c2 < nch ? vj[32 * c2 + lane] : 0.0;
+        reflect2(v, tp[jj], cb, nch, y0, y1);
+      }
+      store_col(A + (long long)l * m, m, nch, y0);
+      store_col(A + (long long)(l + 1) * m, m, nch, y1);
+    }
+    __syncthreads();
+  }
 }
 
 // Householder QR in place of the column-major m x c matrix A (column a at A + a*m), q =
@@ -168,88 +274,45 @@ __device__ void householder_qr(double* A, int m, int c, double* vp, double* tp, 
     }
     return;
   }
+  by_slots(m, [&](auto nc) { qr_panels<decltype(nc)::value>(A, m, c, vp, tp); });
+}
+
+// The kept rows below for at most 32 NC columns, in registers.
+template <int NC>
+__device__ void apply_rows(const double* A, int m, int q, const double* B, int p, double* out, const double* tau) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kRoundThreads / 32;
   const int nch = (m + 31) / 32;
-  for (int j0 = 0; j0 < q; j0 += kPanel) {
-    const int nb = min(kPanel, q - j0), cb = j0 / 32;
-    {  // factor the panel: warp w holds column j0 + w
-      double y[kRegRows];
-      const bool mine = warp < nb;
-      if (mine) load_col(A + (long long)(j0 + warp) * m, m, nch, y);
-      for (int jj = 0; jj < nb; ++jj) {
-        const int j = j0 + jj;
-        double* vj = vp + jj * (32 * kRegRows);
-        if (warp == jj) {
-          double part = 0.0, x0 = 0.0;
+  for (int b0 = 0; b0 < p; b0 += 2 * nw) {
+    // up to 16 rows a round: the first `dbl` warps take two, so that no scheduler holds more
+    // than one above its share
+    const int rem = min(p - b0, 2 * nw), dbl = max(0, rem - nw);
+    const bool two = warp < dbl;
+    const int b = b0 + (two ? 2 * warp : warp + dbl);
+    if (b >= b0 + rem) continue;
+    double y0[NC], y1[NC], v[NC], vn[NC];
 #pragma unroll
-          for (int c2 = 0; c2 < kRegRows; ++c2)
-            if (c2 >= cb && c2 < nch) {
-              const int i = 32 * c2 + lane;
-              if (i >= j) part = fma(y[c2], y[c2], part);
-              if (i == j) x0 = y[c2];
-            }
-          part = warp_sum(part);
-          x0 = __shfl_sync(0xffffffffu, x0, j & 31);
-          double alpha = 0.0, tau = 0.0, inv = 0.0;
-          if (part > 0.0) {
-            const double rn = rsqrt(part);
-            alpha = x0 >= 0.0 ? -(part * rn) : part * rn;
-            tau = fma(fabs(x0), rn, 1.0);  // -v0 / alpha
-            inv = 1.0 / (x0 - alpha);
-          }
-#pragma unroll
-          for (int c2 = 0; c2 < kRegRows; ++c2)
-            if (c2 < nch) {
-              const int i = 32 * c2 + lane;
-              if (i >= j) y[c2] = i == j ? alpha : y[c2] * inv;
-              vj[i] = i > j ? y[c2] : (i == j ? 1.0 : 0.0);
-            }
-          if (lane == 0) tp[jj] = tau;
-        }
-        __syncthreads();
-        if (mine && warp > jj) {
-          double s = 0.0;
-#pragma unroll
-          for (int c2 = 0; c2 < kRegRows; ++c2)
-            if (c2 >= cb && c2 < nch) s = fma(vj[32 * c2 + lane], y[c2], s);
-          s = -tp[jj] * warp_sum(s);
-#pragma unroll
-          for (int c2 = 0; c2 < kRegRows; ++c2)
-            if (c2 >= cb && c2 < nch) y[c2] = fma(s, vj[32 * c2 + lane], y[c2]);
-        }
+    for (int c = 0; c < NC; ++c) {
+      const int i = 32 * c + lane;
+      y0[c] = y1[c] = 0.0;
+      if (c < nch && i < q) {
+        const double sg = A[(long long)i * m + i] < 0.0 ? -1.0 : 1.0;
+        y0[c] = sg * B[(long long)b * q + i];
+        if (two) y1[c] = sg * B[(long long)(b + 1) * q + i];
       }
-      if (mine) store_col(A + (long long)(j0 + warp) * m, m, nch, y);
     }
-    // the panel's reflectors over the trailing columns, two per warp at a time (one per warp when
-    // at most eight are left, so that the last round spreads over all warps)
-    for (int l0 = j0 + nb; l0 < c; l0 += 2 * nw) {
-      const bool pairs = c - l0 > nw;
-      const int l = l0 + (pairs ? 2 * warp : warp);
-      if (l >= c) break;
-      double y0[kRegRows], y1[kRegRows], v[kRegRows];
-      const bool two = pairs && l + 1 < c;
-      if (!two) {
-        load_col(A + (long long)l * m, m, nch, y0);
-        for (int jj = 0; jj < nb; ++jj) {
-          const double* vj = vp + jj * (32 * kRegRows);
+    load_col(A + (long long)(q - 1) * m, m, nch, vn);
+    for (int j = q - 1; j >= 0; --j) {
 #pragma unroll
-          for (int c2 = 0; c2 < kRegRows; ++c2) v[c2] = c2 >= cb && c2 < nch ? vj[32 * c2 + lane] : 0.0;
-          reflect1(v, tp[jj], cb, nch, y0);
-        }
-        store_col(A + (long long)l * m, m, nch, y0);
-        continue;
+      for (int c = 0; c < NC; ++c) {
+        const int i = 32 * c + lane;
+        v[c] = i > j ? vn[c] : (i == j ? 1.0 : 0.0);
       }
-      load_col(A + (long long)l * m, m, nch, y0);
-      load_col(A + (long long)(l + 1) * m, m, nch, y1);
-      for (int jj = 0; jj < nb; ++jj) {
-        const double* vj = vp + jj * (32 * kRegRows);
-#pragma unroll
-        for (int c2 = 0; c2 < kRegRows; ++c2) v[c2] = c2 >= cb && c2 < nch ? vj[32 * c2 + lane] : 0.0;
-        reflect2(v, tp[jj], cb, nch, y0, y1);
-      }
-      store_col(A + (long long)l * m, m, nch, y0);
-      store_col(A + (long long)(l + 1) * m, m, nch, y1);
+      if (j > 0) load_col(A + (long long)(j - 1) * m, m, nch, vn);  // in flight during this reflector
+      if (two) reflect2(v, tau[j], j / 32, nch, y0, y1);
+      else reflect1(v, tau[j], j / 32, nch, y0);
     }
-    __syncthreads();
+    store_col(out + (long long)b * m, m, nch, y0);
+    if (two) store_col(out + (long long)(b + 1) * m, m, nch, y1);
   }
 }
 
@@ -285,39 +348,7 @@ __device__ void apply_q(const double* A, int m, int q, const double* B, int p, d
     }
     return;
   }
-  const int nch = (m + 31) / 32;
-  for (int b0 = 0; b0 < p; b0 += 2 * nw) {
-    // up to 16 rows a round: the first `dbl` warps take two, so that no scheduler holds more
-    // than one above its share
-    const int rem = min(p - b0, 2 * nw), dbl = max(0, rem - nw);
-    const bool two = warp < dbl;
-    const int b = b0 + (two ? 2 * warp : warp + dbl);
-    if (b >= b0 + rem) continue;
-    double y0[kRegRows], y1[kRegRows], v[kRegRows], vn[kRegRows];
-#pragma unroll
-    for (int c = 0; c < kRegRows; ++c) {
-      const int i = 32 * c + lane;
-      y0[c] = y1[c] = 0.0;
-      if (c < nch && i < q) {
-        const double sg = A[(long long)i * m + i] < 0.0 ? -1.0 : 1.0;
-        y0[c] = sg * B[(long long)b * q + i];
-        if (two) y1[c] = sg * B[(long long)(b + 1) * q + i];
-      }
-    }
-    load_col(A + (long long)(q - 1) * m, m, nch, vn);
-    for (int j = q - 1; j >= 0; --j) {
-#pragma unroll
-      for (int c = 0; c < kRegRows; ++c) {
-        const int i = 32 * c + lane;
-        v[c] = i > j ? vn[c] : (i == j ? 1.0 : 0.0);
-      }
-      if (j > 0) load_col(A + (long long)(j - 1) * m, m, nch, vn);  // in flight during this reflector
-      if (two) reflect2(v, tau[j], j / 32, nch, y0, y1);
-      else reflect1(v, tau[j], j / 32, nch, y0);
-    }
-    store_col(out + (long long)b * m, m, nch, y0);
-    if (two) store_col(out + (long long)(b + 1) * m, m, nch, y1);
-  }
+  by_slots(m, [&](auto nc) { apply_rows<decltype(nc)::value>(A, m, q, B, p, out, tau); });
 }
 
 // out (rows x q, row-major) = Wp (rows x c) R^T with R (q x c, upper trapezoid, rows normalised
@@ -325,17 +356,19 @@ __device__ void apply_q(const double* A, int m, int q, const double* B, int p, d
 // owns two columns j and starts its sum at the first a >= j (the zero triangle is skipped); a
 // lane owns one row of each of the tile's 32-row groups, which are shared out evenly over the
 // tiles. 64 steps are staged at a time. wt: kRtK x kRtLd, rt: kRtK x 17 doubles of shared memory.
-__device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m, int q, double* out, double* wt,
-                       double* rt) {
+// NX: the most 32-row groups of a tile here.
+template <int NX>
+__device__ void mul_rt_tiles(const double* Wp, int rows, int c, const double* A, int m, int q, double* out, double* wt,
+                             double* rt) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ng = (rows + 31) / 32, nt = (ng + kRtRows - 1) / kRtRows;
   for (int t = 0; t < nt; ++t) {
     const int g0 = (int)((long long)t * ng / nt), nx = (int)((long long)(t + 1) * ng / nt) - g0;
     const int i0 = 32 * g0, nr = min(32 * nx, rows - i0);
     for (int j0 = 0; j0 < q; j0 += 16) {
-      double acc[kRtRows][2];
+      double acc[NX][2];
 #pragma unroll
-      for (int x = 0; x < kRtRows; ++x) acc[x][0] = acc[x][1] = 0.0;
+      for (int x = 0; x < NX; ++x) acc[x][0] = acc[x][1] = 0.0;
       const int ja = j0 + 2 * warp;
       for (int a0 = j0; a0 < c; a0 += kRtK) {
         const int na = min(kRtK, c - a0);
@@ -358,7 +391,7 @@ __device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m
           for (int aa = max(0, ja - a0); aa < na; ++aa) {
             const double r0 = rt[aa * 17 + 2 * warp], r1 = rt[aa * 17 + 2 * warp + 1];
 #pragma unroll
-            for (int x = 0; x < kRtRows; ++x)
+            for (int x = 0; x < NX; ++x)
               if (x < nx) {
                 const double w = wt[aa * kRtLd + 32 * x + lane];
                 acc[x][0] = fma(w, r0, acc[x][0]);
@@ -367,7 +400,7 @@ __device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m
           }
       }
 #pragma unroll
-      for (int x = 0; x < kRtRows; ++x) {
+      for (int x = 0; x < NX; ++x) {
         const int r = 32 * x + lane;
         if (r < nr) {
           if (ja < q) out[(long long)(i0 + r) * q + ja] = acc[x][0];
@@ -377,6 +410,13 @@ __device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m
     }
   }
   __syncthreads();
+}
+
+__device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m, int q, double* out, double* wt,
+                       double* rt) {
+  if (rows <= 32) mul_rt_tiles<1>(Wp, rows, c, A, m, q, out, wt, rt);
+  else if (rows <= 96) mul_rt_tiles<3>(Wp, rows, c, A, m, q, out, wt, rt);
+  else mul_rt_tiles<kRtRows>(Wp, rows, c, A, m, q, out, wt, rt);
 }
 
 // Cyclic Jacobi eigen-decomposition of the symmetric positive semidefinite s x s matrix S
@@ -392,6 +432,11 @@ __device__ void mul_rt(const double* Wp, int rows, int c, const double* A, int m
 __device__ void jacobi_eig(double* S, double* V, int s, int ld, int* pp, int* pq, double* pc, double* ps, double* red,
                            unsigned short* tri) {
   const int tid = threadIdx.x;
+  if (s == 1) {
+    if (tid == 0) V[0] = 1.0;
+    __syncthreads();
+    return;
+  }
   const int se = s + (s & 1);  // even count; index s is a dummy
   const int np = se / 2, ns = np * (np + 1) / 2;
   double dmax = 0.0;
