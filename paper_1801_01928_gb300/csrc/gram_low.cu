@@ -288,10 +288,12 @@ __device__ void low_left(const GramLowArgs& g, float* sm, int a0, int na, int b0
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
-// Two blocks an SM at R = 4 (64 registers, for large batches) and R = 8 (128), one elsewhere: left to the
-// compiler, R = 8 had 80 registers (100 x 100 pairs of rank 7, d = 6, n = 10: 95 us, now 80) and R = 16 168 (471, now 408).
+// Blocks an SM to leave registers for. Forward us with 1, 2, 3: R = 6, 40 x 40 pairs (d = 6, n = 10) 33, 35, 44
+// and 350 x 350 (d = 5, n = 8) 338, 266, 282; R = 14, 40 x 40 86, -, 90 and 350 x 350 2143, -, 1920 (2112 with 4).
+// Left to the compiler R = 8 had 80 registers for three blocks (100 x 100 of rank 7, d = 6, n = 10: 95, now 80) and
+// R = 16 168 (471, now 408).
 template <int R>
-__global__ void __launch_bounds__(32 * Low<R>::W, R == 4 || R == 8 ? 2 : 1) k_gram_low(const __grid_constant__ GramLowArgs g) {
+__global__ void __launch_bounds__(32 * Low<R>::W, R <= 8 ? 2 : R == 14 ? 3 : 1) k_gram_low(const __grid_constant__ GramLowArgs g) {
   extern __shared__ __align__(16) float sm[];
   const int ntb = (g.B.batch + g.t - 1) / g.t;
   const int a0 = (blockIdx.x / ntb) * g.t, b0 = (blockIdx.x % ntb) * g.t;
@@ -526,7 +528,9 @@ auto low_dispatch(const TTV& A, const TTV& B, F f) {
 //   nothing at all; up to rank 4 every pair of ranks): forward 34 .. 208 against 90 .. 401 and adjoint
 //   92 .. 821 against 250 .. 1856 over batches of 8 x 9 .. 128 x 128, 1.1 to 4.2 times as fast. Forward of
 //   many pairs of ranks 1 and 2 (d = 10, n = 10): 200 x 200 115 against 148, 350 x 350 247 against 225, 500 x
-//   500 445 against 421, 800 x 800 1062 against 1198, so not from 500 to 3000 pairs an SM;
+//   500 445 against 421, 800 x 800 1062 against 1198, so not from 500 to 3000 pairs an SM; ranks 5 and 4 (d = 5, n = 8): 150 x
+//   150 60 against 82, 250 x 250 156 against 123, 350 x 350 265 against 238, 500 x 500 488 against 545, so not
+//   from 200 to 1500;
 //   11 and 12, forward only and up to 46 pairs an SM: 80 x 80 138 against 172, but 90 x 90 of ranks 12 and 9 177
 //   against 168, 128 x 128 with n = 16, d = 4 311 against 290 (two objects of 12 rows a warp); the adjoint 966
 //   against 927 at 96 x 104;
@@ -553,9 +557,10 @@ static bool inner_full(const TTV& A, const TTV& B) {
 
 bool gram_low_supported(const TTV& A, const TTV& B) {
   if (!low_ranks(A, B)) return false;
-  const int hi = std::max(A.rmax, B.rmax);
+  const int hi = std::max(A.rmax, B.rmax), lo = std::min(A.rmax, B.rmax);
   const long long pairs = (long long)A.batch * B.batch, sms = device_sm_count();
   if (hi <= 2) return pairs <= 500 * sms || pairs >= 3000 * sms;
+  if (hi <= 6 && hi > 4 && lo <= 4) return pairs <= 200 * sms || pairs >= 1500 * sms;
   if (hi <= 10) return true;
   if (hi <= 12) return pairs <= 46 * sms;
   return pairs <= 64 * sms || inner_full(A, B);

@@ -17,6 +17,8 @@ torch = pytest.importorskip("torch")
     (275, 276, [2, 3, 2], [1, 2, 2, 1], [1, 2, 1, 1]),    # 500 pairs an SM
     (277, 277, [2, 3, 2], [1, 2, 2, 1], [1, 1, 2, 1]),
     (676, 675, [2, 2], [1, 2, 1], [1, 2, 1]),             # 3000 pairs an SM
+    (174, 174, [2, 3, 2], [1, 5, 4, 1], [1, 4, 4, 1]),    # 200 pairs an SM, sides 5 and 4
+    (175, 174, [2, 3, 2], [1, 5, 4, 1], [1, 4, 4, 1]),
     (83, 84, [3, 2, 2], [1, 12, 11, 1], [1, 11, 12, 1]),  # 46 pairs an SM
     (84, 84, [3, 2, 2], [1, 12, 11, 1], [1, 11, 12, 1]),
     (98, 100, [2, 2, 2], [1, 14, 12, 1], [1, 13, 14, 1]),  # an inner core of rank 12
