@@ -394,11 +394,13 @@ __global__ void __launch_bounds__(kThreads) k_project_core(const __grid_constant
 // and 0.2 to 0.5 us a slice more, with r. Whole calls of 1000 rank-8 objects, d = 8, X of rank r, one kernel
 // against two, us: r = 8: n = 2 301, 105; n = 16 340, 211; r = 16: n = 4 336, 150; n = 16 404, 387; n = 30 541,
 // 720; r = 32: n = 4 394, 259; n = 8 478, 635. With few units an SM the latency of the two kernels counts:
-// 50 objects, r = 8: n = 4 49, 43; n = 8 53, 50; n = 16 53, 58; r = 16: n = 8 53, 53; r = 32: n = 4 58, 64.
+// 50 objects, r = 8: n = 4 49, 43; n = 8 53, 50; n = 16 53, 58; r = 16: n = 8 53, 53; r = 32: n = 4 58, 64; 10
+// objects, r = 8: n = 4 41, 41; n = 8 43, 48.
 static bool small_cores(const TTV& U, int batch, int sms) {
   long long most = 0;
   for (int k = 0; k < U.d; ++k) most = std::max(most, U.osz[k]);
-  return (long long)U.d * batch >= 6LL * sms ? most <= 4096 : most <= 2048 && U.nmax <= 8;
+  const long long units = (long long)U.d * batch;
+  return units >= 2LL * sms && (units >= 6LL * sms ? most <= 4096 : most <= 2048 && U.nmax <= 8);
 }
 
 template <int RU>
