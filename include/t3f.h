@@ -378,7 +378,7 @@ typedef struct {
  * sqrt(G_g[a][a]) in FP64.
  * Scheduling: the objects of every group are ordered by rank into buckets {<=8, <=16, <=32,
  * <=64}; tiles[b] (host int32[4], each in 1..16; NULL or {10, 6, 3, 1} = built-in defaults, larger
- * from 256 objects on) caps the tile side for bucket b. Within a bucket pair, runs of rank-sorted objects grow up to that side while
+ * for large collections) caps the tile side for bucket b. Within a bucket pair, runs of rank-sorted objects grow up to that side while
  * their tile (padded to the run's own largest rank) fits one CTA; the upper triangle of pairs
  * is cut into such tiles, sorted by cost and drained by ONE persistent launch.
  * math (t3f_math): FP32 = CUDA-core FP32 throughout. TF32 (F32 cores) / BF16 (F32 or BF16

@@ -58,25 +58,52 @@ constexpr int kBuckets = 4;
 constexpr int kMmaR[kBuckets] = {16, 16, 32, 64};  // tensor-core padded rank of each bucket
 const int kBucketMax[kBuckets] = {8, 16, 32, 64};
 // Side caps of the forward tiles where the caller gives none. Large tiles read every staged slice
-// more often, small ones even out the SMs of a small collection. FP32 forward, small against large
+// more often, small ones even out the SMs of a small collection, so the large ones from kManyObjects on
+// where they still make two tiles an SM. FP32 forward, small against large
 // caps, groups x objects (ranks 2 .. 64), us: 8 x 64 4587 -> 4103, 7165 -> 6217 and 3751 -> 3207,
-// 6 x 50 2390 -> 2140; below the line 4 x 40 1808 -> 1825, 8 x 16 1204 -> 1210, 1 x 64 712 -> 709.
+// 6 x 50 2390 -> 2140; below the line 4 x 40 1808 -> 1825, 8 x 16 1204 -> 1210, 1 x 64 712 -> 709, 3 x 100 of
+// ranks 2 .. 4 178 -> 213.
 constexpr int kManyObjects = 256;
 const int kDefaultTiles[kBuckets] = {10, 6, 3, 1}, kDefaultTilesMany[kBuckets] = {16, 16, 4, 2};
-// The caps of a call. The small table passed by value is the exported default (the binding's
-// DEFAULT_TILES) and means the same plan as no table at all: a workspace prepared with the one is used
-// with the other.
-inline void tile_caps(int count, const int* tiles, int* tl) {
-  const bool given = tiles && !std::equal(kDefaultTiles, kDefaultTiles + kBuckets, tiles);
-  const int* from = given ? tiles : (count >= kManyObjects ? kDefaultTilesMany : kDefaultTiles);
-  std::copy(from, from + kBuckets, tl);
-}
 
 int sm_count_gg() { return device_sm_count(); }
 
 struct Range {
   int begin, end, R;  // sorted positions [begin, end), padded inner rank
 };
+
+int bucket_of(int r) {
+  for (int b = 0; b < kBuckets; ++b)
+    if (r <= kBucketMax[b]) return b;
+  return -1;
+}
+
+// The caps of a call. The small table passed by value is the exported default (the binding's
+// DEFAULT_TILES) and means the same plan as no table at all: a workspace prepared with the one is used
+// with the other. X's arrays have been looked at as far as d.
+void tile_caps(const t3f_tt_ragged* X, int ngroups, const int* gstart, const int* tiles, int* tl) {
+  const bool given = tiles && !std::equal(kDefaultTiles, kDefaultTiles + kBuckets, tiles);
+  bool many = !given && X->count >= kManyObjects;
+  if (many) {  // tiles of the large caps: the pairs of a group's runs
+    long long n = 0, ro = 0;
+    int o = 0;
+    for (int g = 0; g < ngroups; ++g) {
+      int cnt[kBuckets] = {};
+      for (; o < gstart[g + 1] && o < X->count; ++o) {
+        int r = 1;
+        for (int k = 0; k <= X->d[o]; ++k) r = std::max(r, (int)X->ranks[ro + k]);
+        ro += X->d[o] + 1;
+        if (const int b = bucket_of(r); b >= 0) ++cnt[b];
+      }
+      long long runs = 0;
+      for (int b = 0; b < kBuckets; ++b) runs += (cnt[b] + kDefaultTilesMany[b] - 1) / kDefaultTilesMany[b];
+      n += runs * (runs + 1) / 2;
+    }
+    many = n >= 2LL * sm_count_gg();
+  }
+  const int* from = given ? tiles : (many ? kDefaultTilesMany : kDefaultTiles);
+  std::copy(from, from + kBuckets, tl);
+}
 
 struct Plan {
   int count = 0, ngroups = 0, dmax = 0, nitems = 0;
@@ -112,12 +139,6 @@ struct Plan {
       o_titems, total;
 };
 
-int bucket_of(int r) {
-  for (int b = 0; b < kBuckets; ++b)
-    if (r <= kBucketMax[b]) return b;
-  return -1;
-}
-
 inline size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
 t3f_status build_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, const int* tiles, Plan* P) {
@@ -125,8 +146,10 @@ t3f_status build_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, co
   if (X->count < 1 || ngroups < 1 || !gstart) return T3F_ERR_ARG;
   if (X->dtype != T3F_F32 && X->dtype != T3F_BF16) return T3F_ERR_DTYPE;
   if (gstart[0] != 0 || gstart[ngroups] != X->count) return T3F_ERR_SHAPE;
+  for (int o = 0; o < X->count; ++o)
+    if (X->d[o] < 1 || X->d[o] > T3F_MAX_D) return T3F_ERR_SHAPE;
   int tl[kBuckets];
-  tile_caps(X->count, tiles, tl);
+  tile_caps(X, ngroups, gstart, tiles, tl);
   for (int b = 0; b < kBuckets; ++b)
     if (tl[b] < 1 || tl[b] > 16) return T3F_ERR_ARG;
   const int cnt = X->count;
@@ -577,7 +600,7 @@ t3f_status get_plan(const t3f_tt_ragged* X, int ngroups, const int* gstart, cons
       key.reserve(16 + 3 * (size_t)X->count + 2 * sd + X->count + ngroups);
       key.insert(key.end(), head, head + 4);
       int tl[kBuckets];
-      tile_caps(X->count, tiles, tl);
+      tile_caps(X, ngroups, gstart, tiles, tl);
       key.insert(key.end(), tl, tl + kBuckets);
       key.insert(key.end(), gstart, gstart + ngroups + 1);
       key.insert(key.end(), X->d, X->d + X->count);
