@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_bwd(const __grid_cons
 // Bound by shared-memory wavefronts (a chain step reads R^2 slice values per tuple for as many
 // multiply-adds). 10^6 tuples, d = 10, n = 10, r = 8: 529 us with one thread per tuple walking both
 // chains through its own slices, 422 us with the chains on two threads (shared-memory pipe 71 %
-// busy, 5.8 wavefronts a request), 405 us in bucket order (66 %); with two sets of slices (the Riemannian
-// form) 591 -> 462 -> 452 us. r = 4, 1.5 10^6 tuples: 284 us with one thread per tuple, 365 in bucket order
+// busy, 5.8 wavefronts a request), 390 us in bucket order (65 %); with two sets of slices (the Riemannian
+// form) 591 -> 462 -> 433 us. r = 4, 1.5 10^6 tuples: 284 us with one thread per tuple, 365 in bucket order
 // with half the tuples in flight, now 236.
 struct CompletionArgs {
   GatherArgs g;

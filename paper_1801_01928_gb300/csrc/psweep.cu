@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(256) k_pgrad(const __grid_constant__ PGradFast
   const int tile = blockIdx.x % a.ntiles, k = blockIdx.x / a.ntiles;
   const int tid = threadIdx.x;
   const int grp = tid / G, qa = tid % G;
-  const int h = grp / J, ol = grp % J;  // (threads = J SPLIT G, a multiple of 32)
+  const int h = grp / J, ol = grp % J;  // (threads = J SPLIT G: whole warps where G > 1 and there are shuffles, 16 at the least)
   const int obj = tile * J + ol;
   const bool valid = obj < Z.batch;
   const int r0 = a.ra[k], r1 = a.ra[k + 1], z0 = Z.r[k], z1 = Z.r[k + 1], n = Z.n[k];

@@ -18,9 +18,9 @@
 // and then passes the panel's eight reflectors over two trailing columns at a time held in
 // registers (one read and one write of a column per panel instead of per reflector; two
 // columns share their lane reductions); W R^T runs the triangle only. 100 objects of rank 100
-// (d = 10, n = 4) to rank 10: 57.0 ms with Q formed column by column through L2, 28.1 ms this
-// way, the FP64 pipe of the 100 busy SMs 70 % active (QR 43 %, W R^T 17 %, Jacobi 27 %, reflectors
-// on the kept rows 10 % of the time).
+// (d = 10, n = 4) to rank 10: 57.0 ms with Q formed column by column through L2, 27.4 ms this
+// way, the FP64 pipe of the 100 busy SMs 62 % active (28.1 ms and 70 % with one register count for all
+// column heights, of which the QR took 43 %, W R^T 17 %, Jacobi 27 %, reflectors on the kept rows 10 %).
 #include <math.h>
 #include <string.h>
 
